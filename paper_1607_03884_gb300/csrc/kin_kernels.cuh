@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 
 #include "../../include/kin.h"
+#include "kin_coop.cuh"
 #include "kin_radau.cuh"
 #include "kin_warp.cuh"
 
@@ -214,6 +215,61 @@ __global__ void KIN_THREAD_BOUNDS k_integrate_queue(KernelArgs a) {
   }
 }
 
+// PLAIN on a small batch: one state per block (kin_coop.cuh).  Eight blocks
+// per SM cap the registers at 80; a batch of 1024 is seven states per SM.
+template <typename LT, bool FDJ>
+__global__ void __launch_bounds__(COOP_NT, 8) k_integrate_coop(KernelArgs a) {
+  extern __shared__ __align__(16) unsigned char coop_smem[];
+  CoopState<LT> &c = *reinterpret_cast<CoopState<LT> *>(coop_smem);
+  const MechView m = make_view(a.L, a.tab, a.itab);
+  const int nr = m.nr, N = m.ns, tid = threadIdx.x;
+  CoopTail<LT> t;
+  t.q = reinterpret_cast<double *>(coop_smem + (sizeof(CoopState<LT>) + 15) / 16 * 16);
+  t.pkf = reinterpret_cast<LT *>(t.q + 3 * nr);
+  t.pkr = t.pkf + nr;
+  t.uJ = t.pkf + 2 * nr;
+  t.sJ = t.pkf + 3 * nr;
+  t.tJ = t.pkf + 4 * nr;
+  t.occ = reinterpret_cast<int *>(t.pkf + 5 * nr);
+  if (tid == 0) c.outcome = (int)state_of(a, blockIdx.x);
+  __syncthreads();
+  const int64_t i = c.outcome, n = a.rp.n;
+  if (i < 0) return;
+  Coop<LT> w{m, c, t, a.P[i]};
+  if (tid < N) c.y[tid] = tid == 0 ? a.T[i] : a.Y[(int64_t)(tid - 1) * n + i];
+  w.build_lists();  // ends with a barrier
+  // every attempt ends the loop or counts a step; max_steps bounds it
+  bool done = w.template init<FDJ>(a.rp, i);
+  while (!done) done = w.template step<FDJ>(a.rp, i);
+  __syncthreads();
+  if (tid < N) (tid == 0 ? a.T[i] : a.Y[(int64_t)(tid - 1) * n + i]) = c.y[tid];
+  if (tid == 0) {
+    const StepState &s = c.s;
+    double sum = 0.0;
+    for (int k = 0; k < N - 1; ++k) sum += c.y[1 + k];
+    a.Y[(int64_t)(N - 1) * n + i] = 1.0 - sum;
+    if (a.status) a.status[i] = s.status;
+    const int32_t v[8] = {s.nstep, s.naccpt, s.nrejct, s.nfcn, s.njac, s.ndec, s.nsol, s.status};
+    for (int q = 0; q < 8; ++q) {
+      if (a.counters) a.counters[(int64_t)q * n + i] = v[q];
+      if (q < 7) atomicAdd(a.totals + q, (unsigned long long)v[q]);
+    }
+    if (s.status) atomicAdd(a.totals + 7, 1ull);
+    atomicMax(a.totals + 8, (unsigned long long)s.nstep);
+  }
+}
+
+// PLAIN batches of at most this many states go to k_integrate_coop: its time
+// grows with the batch, the per-thread kernel's is flat (a chain of FP64
+// latencies) until its warps fill the chip.  H2, dt = 1e-6 / 1e-4 s, ms,
+// coop against per thread: FP64 2048: 40 / 60 against 156 / 166, 6144:
+// 110 / 169 against 158 / 174, 8192: 145 / 226 against 168 / 171; FP32 2048:
+// 26 / 36 against 121 / 126, 6144: 68 / 105 against 122 / 130, 8192: 91 / 141
+// against 127 / 130.  Both give the same bits.
+constexpr int64_t coop_max_n(size_t lt) { return lt == sizeof(double) ? 6144 : 7168; }
+// ... and a mechanism whose reaction tail leaves several blocks per SM
+constexpr size_t COOP_MAX_SMEM = 64 * 1024;
+
 // WARP layout: one state per group of L lanes; groups pop states from the
 // atomic queue.
 // Register cap of the WARP kernels (0: the compiler's choice under the
@@ -348,6 +404,17 @@ int launch_t(const KernelArgs &a, const kin_options &o, cudaStream_t st, int sms
   if (block > 64 || block % 32) return KIN_ERR_INVALID_ARG;
   const size_t sm = thread_smem_bytes<MAXN>(a.L, block);
   const int carve = KIN_THREAD_CARVEOUT;  // percent of the unified L1 given to shared memory
+  if constexpr (MAXN <= COOP_CAP) {
+    const size_t smc = coop_smem_bytes<LT>(a.L.nr);
+    if (o.layout == KIN_LAYOUT_PLAIN && a.rp.n <= coop_max_n(sizeof(LT)) &&
+        smc <= COOP_MAX_SMEM) {
+      auto kern = k_integrate_coop<LT, FDJ>;
+      KIN_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smc));
+      kern<<<(unsigned)a.rp.n, COOP_NT, smc, st>>>(a);
+      KIN_CUDA_TRY(cudaGetLastError());
+      return KIN_OK;
+    }
+  }
   if (o.layout == KIN_LAYOUT_PLAIN) {
     auto kern = k_integrate_plain<MAXN, LT, FDJ>;
     KIN_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
