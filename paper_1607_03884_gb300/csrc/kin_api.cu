@@ -408,6 +408,8 @@ int kin::build_tables(const kin_mech_desc *d, MechLayout &L, std::vector<double>
       tp[6] = f[6];
       troe_idx = tr++;
     }
+    L.nslots += nre + npr;
+    L.nterms += (nre + npr) * (nre + npr + ne);
     it[L.imeta + i] = t | (nre << 2) | (npr << 4) | (ne << 8) | (troe_idx << 16);
     dt[L.dnu + i] = (double)(npr - nre);
   }

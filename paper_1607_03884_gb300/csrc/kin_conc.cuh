@@ -523,6 +523,35 @@ struct ConcSys {
                                       bool wantJ) const {
     return conc_chem<L, LT>(*m, *cv, b, P, y, f, wantJ);
   }
+  __device__ __forceinline__ int chem3(const WarpBuf<LT> &b, double P, const WV &y1, const WV &y2,
+                                       const WV &y3, WV &f1, WV &f2, WV &f3) const {
+    int bad = chem(b, P, y1, f1, false);
+    bad |= chem(b, P, y2, f2, false);
+    bad |= chem(b, P, y3, f3, false);
+    return bad;
+  }
+  __device__ __forceinline__ int jat(const WarpBuf<LT> &b, int i, int j) const {
+    return i * b.ld + j;
+  }
+  __device__ __forceinline__ void solve_both(const WarpBuf<LT> &b, WV &x, WV &xr, WV &xi) const {
+    solve_real(b, x);
+    solve_cplx(b, xr, xi);
+  }
+  // J x with x gathered by shuffles (element j on lane j % L, slot j / L)
+  __device__ __forceinline__ void jac_times(const WarpBuf<LT> &b, const WV &x, WV &out) const {
+    constexpr int WR = Grp<L>::WR;
+    const int lane = Grp<L>::lane(), N = n();
+#pragma unroll
+    for (int r = 0; r < WR; ++r) out.v[r] = 0.0;
+    for (int j = 0; j < N; ++j) {
+      const double xj = elem<L>(x, j);
+#pragma unroll
+      for (int r = 0; r < WR; ++r) {
+        const int i = lane + L * r;
+        if (i < N) out.v[r] += double(b.J[jat(b, i, j)]) * xj;
+      }
+    }
+  }
   __device__ __forceinline__ int factor(const WarpBuf<LT> &b, double h) const {
     return conc_factor<L, LT>(*cv, b, h);
   }

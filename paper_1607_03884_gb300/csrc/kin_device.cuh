@@ -34,6 +34,9 @@ struct MechLayout {
   // int-table offsets
   int islot, imeta, ieff0, itroe, ieffsp;
   int icsr0, icsr;  // species -> (reaction, net nu) lists: offsets [ns+1], entries
+  // sizes of the team kernels' Jacobian: reaction slots in all; species rows
+  // x (slots + efficiencies) over all reactions (the rows' terms)
+  int nslots, nterms;
 };
 
 // per-species coefficient blocks (two ranges each):
@@ -134,8 +137,12 @@ __device__ __forceinline__ double poly_dcp(const double *c, double T) {
 // ---------------------------------------------------------------------------
 constexpr int EXP_TAB = 256;
 
+// out of line: a copy of the library's code at every call of kexp is
+// instruction-cache space the kernels need
+static __device__ __noinline__ double exp_far(double x) { return exp(x); }
+
 __device__ __forceinline__ double kexp(double x, const double *tab) {
-  if ((__double2hiint(x) & 0x7fffffff) >= 0x4085E000) return exp(x);  // |x| >= 700, NaN
+  if ((__double2hiint(x) & 0x7fffffff) >= 0x4085E000) return exp_far(x);  // |x| >= 700, NaN
   const double inv = 0x1.71547652b82fep+8;    // 256 / ln 2
   const double hi = 0x1.62e42ff000000p-9;     // ln2/256, 29 significant bits
   const double lo = -0x1.718432a1b0e26p-43;   // ln2/256 - hi

@@ -7,6 +7,7 @@
 #include "../../include/kin.h"
 #include "kin_coop.cuh"
 #include "kin_radau.cuh"
+#include "kin_team.cuh"
 #include "kin_warp.cuh"
 
 namespace kin {
@@ -270,6 +271,43 @@ constexpr int64_t coop_max_n(size_t lt) { return lt == sizeof(double) ? 6144 : 7
 // ... and a mechanism whose reaction tail leaves several blocks per SM
 constexpr size_t COOP_MAX_SMEM = 64 * 1024;
 
+// a finished state's vector, status and counters, from its group of L lanes
+template <int L>
+__device__ __forceinline__ void store_lanes(const WVecT<Grp<L>::WR> &y, const StepState &s,
+                                            const KernelArgs &a, int N, int64_t idx) {
+  using G = Grp<L>;
+  constexpr int WR = G::WR;
+  const int lane = G::lane();
+  const int64_t n = a.rp.n;
+  double sum = 0.0;
+#pragma unroll
+  for (int r = 0; r < WR; ++r) {
+    const int g = lane + L * r;
+    if (g == 0) a.T[idx] = y.v[r];
+    if (g >= 1 && g < N) {
+      a.Y[(int64_t)(g - 1) * n + idx] = y.v[r];
+      sum += y.v[r];
+    }
+  }
+  sum = G::sum(sum);
+  if (lane == 0) {
+    a.Y[(int64_t)(N - 1) * n + idx] = 1.0 - sum;
+    if (a.status) a.status[idx] = s.status;
+    if (a.counters) {
+      const int32_t c[8] = {s.nstep, s.naccpt, s.nrejct, s.nfcn, s.njac, s.ndec, s.nsol,
+                            s.status};
+      for (int q = 0; q < 8; ++q) a.counters[(int64_t)q * n + idx] = c[q];
+    }
+    const unsigned long long c7[7] = {
+        (unsigned long long)s.nstep, (unsigned long long)s.naccpt, (unsigned long long)s.nrejct,
+        (unsigned long long)s.nfcn,  (unsigned long long)s.njac,   (unsigned long long)s.ndec,
+        (unsigned long long)s.nsol};
+    for (int q = 0; q < 7; ++q) atomicAdd(a.totals + q, c7[q]);
+    if (s.status) atomicAdd(a.totals + 7, 1ull);
+    atomicMax(a.totals + 8, (unsigned long long)s.nstep);
+  }
+}
+
 // WARP layout: one state per group of L lanes; groups pop states from the
 // atomic queue.
 // Register cap of the WARP kernels (0: the compiler's choice under the
@@ -319,33 +357,7 @@ __global__ void KIN_WARP_BOUNDS k_integrate_lanes(KernelArgs a) {
     // every attempt ends the loop or counts a step; max_steps bounds it
     bool done = warp_init<L, LT, FDJ>(m, b, P, w, s, a.rp, idx);
     while (!done) done = warp_step<L, LT, FDJ>(m, b, P, w, s, a.rp, idx);
-    double sum = 0.0;
-#pragma unroll
-    for (int r = 0; r < WR; ++r) {
-      const int g = lane + L * r;
-      if (g == 0) a.T[idx] = w.y.v[r];
-      if (g >= 1 && g < N) {
-        a.Y[(int64_t)(g - 1) * n + idx] = w.y.v[r];
-        sum += w.y.v[r];
-      }
-    }
-    sum = G::sum(sum);
-    if (lane == 0) {
-      a.Y[(int64_t)(N - 1) * n + idx] = 1.0 - sum;
-      if (a.status) a.status[idx] = s.status;
-      if (a.counters) {
-        const int32_t c[8] = {s.nstep, s.naccpt, s.nrejct, s.nfcn, s.njac, s.ndec, s.nsol,
-                              s.status};
-        for (int q = 0; q < 8; ++q) a.counters[(int64_t)q * n + idx] = c[q];
-      }
-      const unsigned long long c7[7] = {
-          (unsigned long long)s.nstep, (unsigned long long)s.naccpt, (unsigned long long)s.nrejct,
-          (unsigned long long)s.nfcn,  (unsigned long long)s.njac,   (unsigned long long)s.ndec,
-          (unsigned long long)s.nsol};
-      for (int q = 0; q < 7; ++q) atomicAdd(a.totals + q, c7[q]);
-      if (s.status) atomicAdd(a.totals + 7, 1ull);
-      atomicMax(a.totals + 8, (unsigned long long)s.nstep);
-    }
+    store_lanes<L>(w.y, s, a, N, idx);
     G::sync();
   }
 }
@@ -354,6 +366,88 @@ __global__ void KIN_WARP_BOUNDS k_integrate_lanes(KernelArgs a) {
 __host__ __device__ inline size_t lanes_smem_bytes(const MechLayout &L_, int lanes, size_t lt,
                                                    int warps) {
   return (size_t)warps * (32 / lanes) * warp_buf_bytes(L_.ns, L_.nr, lt);
+}
+
+// WARP layout with 32 lanes: a state per team of three warps (kin_team.cuh),
+// up to four teams per block, one block per SM.
+template <typename LT, bool FDJ>
+__global__ void __launch_bounds__(TEAM_MAX *TEAM_NT, 1) k_integrate_team(KernelArgs a) {
+  using G = Grp<32>;
+  extern __shared__ __align__(16) unsigned char team_smem[];
+  const MechView m = make_view(a.L, a.tab, a.itab);
+  const int N = m.ns, lane = G::lane(), warp = (int)(threadIdx.x / 32);
+  const int team = warp / TEAM_WARPS, wt = warp % TEAM_WARPS;
+  const int64_t n = a.rp.n;
+  const HotTables h = stage_hot(m, a.L, team_smem);  // ends with a block barrier
+  const size_t tb = team_bytes(a.L, N, sizeof(LT));
+  const int64_t slot = (int64_t)blockIdx.x * (blockDim.x / TEAM_NT) + team;  // < gslots (launch)
+  const TeamBuf<LT> t = carve_team<LT>(
+      a.L, team_smem + hot_bytes(a.L) + team * tb, team, N,
+      reinterpret_cast<unsigned char *>(a.gscratch) +
+          slot * (int64_t)warp_slot_mats(sizeof(LT)) * N * (N + 1) * (int64_t)sizeof(LT));
+  const TeamMassFrac<LT> f{m, h, t};
+  if (wt != 0) {  // workers: a part of each command until the leader is done
+    for (;;) {
+      named_sync(t.bar, TEAM_NT);
+      const int cmd = t.ctl->cmd;
+      if (cmd == TEAM_QUIT) return;
+      team_exec<LT>(cmd, wt, f);
+      named_sync(t.bar, TEAM_NT);
+    }
+  }
+  const TeamSys<LT, TeamMassFrac<LT>> sys{f};
+  WarpBuf<LT> b{};
+  b.J = t.J;
+  unsigned long long *queue = a.totals + 9;
+  WStateT<2> w;
+  StepState s;
+  for (;;) {
+    unsigned long long q = 0;
+    if (lane == 0) q = atomicAdd(queue, 1ull);
+    q = G::bcast(q, 0);
+    if (q >= (unsigned long long)n) break;
+    int64_t idx = 0;
+    if (lane == 0) idx = state_of(a, (int64_t)q);
+    idx = G::bcast(idx, 0);
+    if (idx < 0) continue;
+    const double P = a.P[idx];
+    if (lane == 0) t.ctl->P = P;
+    __syncwarp();
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+      const int g = lane + 32 * r;
+      w.y.v[r] = (g == 0) ? a.T[idx] : (g < N ? a.Y[(int64_t)(g - 1) * n + idx] : 0.0);
+    }
+    // every attempt ends the loop or counts a step; max_steps bounds it
+    bool done = warp_init_sys<32, LT, FDJ>(sys, b, P, w, s, a.rp, idx);
+    while (!done) done = warp_step_sys<32, LT, FDJ>(sys, b, P, w, s, a.rp, idx);
+    store_lanes<32>(w.y, s, a, N, idx);
+  }
+  sys.post(TEAM_QUIT);
+}
+
+template <typename LT, bool FDJ>
+int launch_team(const KernelArgs &a, cudaStream_t st, int sms, bool &fits) {
+  if (!a.gscratch || a.gslots < 1) return KIN_ERR_UNSUPPORTED;
+  const size_t budget = 227 * 1024;
+  const size_t hot = hot_bytes(a.L), tb = team_bytes(a.L, a.L.ns, sizeof(LT));
+  // 12-bit reaction numbers and 15-bit derivative indices in the staged lists
+  fits = hot + tb <= budget && a.L.nr < 4096 && a.L.nslots + a.L.neff < 32768;
+  if (!fits) return KIN_OK;
+  int64_t teams = (int64_t)((budget - hot) / tb);
+  teams = teams < TEAM_MAX ? teams : TEAM_MAX;
+  const int64_t want = (a.rp.n + sms - 1) / sms;  // a small batch spreads over the SMs
+  teams = teams < want ? teams : want;
+  int64_t grid = (a.rp.n + teams - 1) / teams;
+  grid = grid < sms ? grid : sms;
+  if (grid * teams > a.gslots) grid = a.gslots / teams;
+  if (grid < 1) return KIN_ERR_UNSUPPORTED;
+  const size_t sm = hot + teams * tb;
+  auto kern = k_integrate_team<LT, FDJ>;
+  KIN_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+  kern<<<(unsigned)grid, (unsigned)(teams * TEAM_NT), sm, st>>>(a);
+  KIN_CUDA_TRY(cudaGetLastError());
+  return KIN_OK;
 }
 
 template <int L, typename LT, bool FDJ>
@@ -395,18 +489,22 @@ int launch_t(const KernelArgs &a, const kin_options &o, cudaStream_t st, int sms
   if (o.layout == KIN_LAYOUT_WARP) {
     if constexpr (MAXN == 64) {
       if (a.L.ns > 63) return KIN_ERR_UNSUPPORTED;
-      return launch_lanes<32, LT, FDJ>(a, st, sms);
+      bool fits = false;
+      const int rc = launch_team<LT, FDJ>(a, st, sms, fits);
+      if (fits) return rc;
+      // more reactions than a team's shared memory holds: a state per thread
     } else {
       return KIN_ERR_UNSUPPORTED;
     }
   }
+  const bool plain = o.layout != KIN_LAYOUT_QUEUE;
   const int block = o.block > 0 ? o.block : 64;
   if (block > 64 || block % 32) return KIN_ERR_INVALID_ARG;
   const size_t sm = thread_smem_bytes<MAXN>(a.L, block);
   const int carve = KIN_THREAD_CARVEOUT;  // percent of the unified L1 given to shared memory
   if constexpr (MAXN <= COOP_CAP) {
     const size_t smc = coop_smem_bytes<LT>(a.L.nr);
-    if (o.layout == KIN_LAYOUT_PLAIN && a.rp.n <= coop_max_n(sizeof(LT)) &&
+    if (plain && a.rp.n <= coop_max_n(sizeof(LT)) &&
         smc <= COOP_MAX_SMEM) {
       auto kern = k_integrate_coop<LT, FDJ>;
       KIN_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smc));
@@ -415,7 +513,7 @@ int launch_t(const KernelArgs &a, const kin_options &o, cudaStream_t st, int sms
       return KIN_OK;
     }
   }
-  if (o.layout == KIN_LAYOUT_PLAIN) {
+  if (plain) {
     auto kern = k_integrate_plain<MAXN, LT, FDJ>;
     KIN_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
     KIN_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, carve));

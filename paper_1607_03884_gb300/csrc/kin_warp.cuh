@@ -811,8 +811,10 @@ __device__ int warp_factor(int N, const WarpBuf<LT> &b, double h) {
 
 // The system a group integrates, as a policy of the step drivers below: its
 // size n(), the absolute tolerance's factor per element atol_w(), right-hand
-// side (and Jacobian) chem(), factorisation of E1 and E2 factor(), and the
-// two solves.  MassFracSys is the mass-fraction reactor
+// side (and Jacobian) chem(), the right-hand sides at three points chem3(),
+// factorisation of E1 and E2 factor(), the two solves (and both of a Newton
+// iteration, solve_both()), and where the stored Jacobian keeps entry (i, j),
+// jat().  MassFracSys is the mass-fraction reactor
 // with dense Newton matrices and partial pivoting; kin_conc.cuh adds the
 // concentration-based form with a sparse LU.
 template <int L, typename LT>
@@ -826,8 +828,37 @@ struct MassFracSys {
                                       bool wantJ) const {
     return warp_chem<L, LT>(*m, b, P, y, f, wantJ);
   }
+  __device__ __forceinline__ int chem3(const WarpBuf<LT> &b, double P, const WV &y1, const WV &y2,
+                                       const WV &y3, WV &f1, WV &f2, WV &f3) const {
+    int bad = chem(b, P, y1, f1, false);
+    bad |= chem(b, P, y2, f2, false);
+    bad |= chem(b, P, y3, f3, false);
+    return bad;
+  }
+  __device__ __forceinline__ int jat(const WarpBuf<LT> &b, int i, int j) const {
+    return i * b.ld + j;
+  }
+  // J x with x gathered by shuffles (element j on lane j % L, slot j / L)
+  __device__ __forceinline__ void jac_times(const WarpBuf<LT> &b, const WV &x, WV &out) const {
+    constexpr int WR = Grp<L>::WR;
+    const int lane = Grp<L>::lane(), N = n();
+#pragma unroll
+    for (int r = 0; r < WR; ++r) out.v[r] = 0.0;
+    for (int j = 0; j < N; ++j) {
+      const double xj = elem<L>(x, j);
+#pragma unroll
+      for (int r = 0; r < WR; ++r) {
+        const int i = lane + L * r;
+        if (i < N) out.v[r] += double(b.J[jat(b, i, j)]) * xj;
+      }
+    }
+  }
   __device__ __forceinline__ int factor(const WarpBuf<LT> &b, double h) const {
     return warp_factor<L, LT>(m->ns, b, h);
+  }
+  __device__ __forceinline__ void solve_both(const WarpBuf<LT> &b, WV &x, WV &xr, WV &xi) const {
+    solve_real(b, x);
+    solve_cplx(b, xr, xi);
   }
   __device__ __forceinline__ void solve_real(const WarpBuf<LT> &b, WV &x) const {
     warp_solve_real<L, LT>(m->ns, b.ld, b.E1, b.ip1, b.v1, x);
@@ -897,23 +928,12 @@ __device__ void warp_solve_e1(const Sys &sys, const WarpBuf<LT> &b, double h,
     sys.solve_real(b, x);
     return;
   }
-  const int lane = Grp<L>::lane();
   const WVecT<WR> rhs = x;
   sys.solve_real(b, x);
   // residual r = rhs - (gamma/h x - J x)
   const double fac1 = RC.gam / h;
   WVecT<WR> res;
-#pragma unroll
-  for (int r = 0; r < WR; ++r) res.v[r] = 0.0;
-  // J x with x gathered by shuffles (element j on lane j % L, slot j / L)
-  for (int j = 0; j < N; ++j) {
-    const double xj = elem<L>(x, j);
-#pragma unroll
-    for (int r = 0; r < WR; ++r) {
-      const int i = lane + L * r;
-      if (i < N) res.v[r] += double(b.J[i * b.ld + j]) * xj;
-    }
-  }
+  sys.jac_times(b, x, res);
 #pragma unroll
   for (int r = 0; r < WR; ++r) res.v[r] = rhs.v[r] - fac1 * x.v[r] + res.v[r];
   sys.solve_real(b, res);
@@ -988,19 +1008,28 @@ __device__ bool warp_step_sys(const Sys &sys, const WarpBuf<LT> &b, double P,
         const double fn = wrms_w<L>(N, w.f0, w.scal);
         const double mininc =
             (fn != 0.0) ? 1000.0 * fabs(s.h) * 2.220446049250313e-16 * N * fn : 1.0;
-        for (int j = 0; j < N; ++j) {
-          const double yj = elem<L>(w.y, j);
-          const double sj = elem<L>(w.scal, j);
-          const double inc = fmax(1.4901161193847656e-08 * fabs(yj), mininc * sj);
+        for (int j0 = 0; j0 < N; j0 += 3) {  // three columns at a time
+          WVecT<WR> u[3], fj[3];
+          double inc[3];
 #pragma unroll
-          for (int r = 0; r < WR; ++r) w.u.v[r] = w.y.v[r];
-          if (lane == (j & (L - 1))) slot_set<WR>(w.u, j / L, yj + inc);
-          rc |= sys.chem(b, P, w.u, w.fu, false);
+          for (int q = 0; q < 3; ++q) {
+            const int j = j0 + q < N ? j0 + q : N - 1;
+            const double yj = elem<L>(w.y, j);
+            const double sj = elem<L>(w.scal, j);
+            inc[q] = fmax(1.4901161193847656e-08 * fabs(yj), mininc * sj);
 #pragma unroll
-          for (int r = 0; r < WR; ++r) {
-            const int i = lane + L * r;
-            if (i < N) b.J[i * b.ld + j] = LT((w.fu.v[r] - w.f0.v[r]) / inc);
+            for (int r = 0; r < WR; ++r) u[q].v[r] = w.y.v[r];
+            if (lane == (j & (L - 1))) slot_set<WR>(u[q], j / L, yj + inc[q]);
           }
+          rc |= sys.chem3(b, P, u[0], u[1], u[2], fj[0], fj[1], fj[2]);
+#pragma unroll
+          for (int q = 0; q < 3; ++q)
+#pragma unroll
+            for (int r = 0; r < WR; ++r) {
+              const int i = lane + L * r;
+              if (i < N && j0 + q < N)
+                b.J[sys.jat(b, i, j0 + q)] = LT((fj[q].v[r] - w.f0.v[r]) / inc[q]);
+            }
         }
         G::sync();
         s.nfcn += N;
@@ -1058,16 +1087,14 @@ __device__ bool warp_step_sys(const Sys &sys, const WarpBuf<LT> &b, double P,
       outcome = 3;
       break;
     }
-    int bad = 0;
+    WVecT<WR> u2, u3;
 #pragma unroll
-    for (int r = 0; r < WR; ++r) w.u.v[r] = w.y.v[r] + w.z1.v[r];
-    bad |= sys.chem(b, P, w.u, w.F1, false);
-#pragma unroll
-    for (int r = 0; r < WR; ++r) w.u.v[r] = w.y.v[r] + w.z2.v[r];
-    bad |= sys.chem(b, P, w.u, w.F2, false);
-#pragma unroll
-    for (int r = 0; r < WR; ++r) w.u.v[r] = w.y.v[r] + w.z3.v[r];
-    bad |= sys.chem(b, P, w.u, w.fu, false);
+    for (int r = 0; r < WR; ++r) {
+      w.u.v[r] = w.y.v[r] + w.z1.v[r];
+      u2.v[r] = w.y.v[r] + w.z2.v[r];
+      u3.v[r] = w.y.v[r] + w.z3.v[r];
+    }
+    const int bad = sys.chem3(b, P, w.u, u2, u3, w.F1, w.F2, w.fu);
     s.nfcn += 3;
     if (bad) {
       outcome = 3;
@@ -1083,8 +1110,7 @@ __device__ bool warp_step_sys(const Sys &sys, const WarpBuf<LT> &b, double P,
       w.z2.v[r] = g2 - (alphn * w.w2.v[r] - betan * w.w3.v[r]);
       w.z3.v[r] = g3 - (betan * w.w2.v[r] + alphn * w.w3.v[r]);
     }
-    sys.solve_real(b, w.z1);
-    sys.solve_cplx(b, w.z2, w.z3);
+    sys.solve_both(b, w.z1, w.z2, w.z3);
     double sum = 0.0;
 #pragma unroll
     for (int r = 0; r < WR; ++r) {
