@@ -18,6 +18,7 @@
 // the 3 N stage increments, de-standardised.
 #include <cuda.h>
 #include <cudaTypedefs.h>
+#include <cooperative_groups.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -129,6 +130,42 @@ __device__ __forceinline__ void tc_stage_row(unsigned char *dst, const __nv_bflo
     d[e] = (row_ok && gk + e < ke) ? src_row[(int64_t)(gk + e) * sk] : __float2bfloat16(0.0f);
 }
 
+// A 128 x 64 slice of an operand contiguous in its rows (element (r, k) at
+// src[k * sk + r]): a thread loads eight rows at k and k + 1 and stores the
+// eight (k, k + 1) pairs; the pairs' order is rotated by lane, so a warp's
+// 32-bit stores fall into 32 banks.  rows: rows left in the matrix.
+__device__ __forceinline__ void tc_stage_t(unsigned char *dst, const __nv_bfloat16 *src, int64_t sk,
+                                           int rows, int k0, int ke) {
+#pragma unroll
+  for (int it = 0; it < (TC_BM / 8) * (TC_BK / 2) / TC_THREADS; ++it) {
+    const int e = it * TC_THREADS + (int)threadIdx.x;
+    // lanes: four k pairs of a core matrix, eight row groups; then the rest
+    const int kp = (e & 3) + 4 * ((e >> 6) & 7), rg = (e >> 2) & 15;
+    const int k = 2 * kp, gk = k0 + k, r = 8 * rg;
+    uint4 a = {0, 0, 0, 0}, b = {0, 0, 0, 0};
+    if (r < rows) {
+      if (gk < ke) a = *reinterpret_cast<const uint4 *>(src + (int64_t)gk * sk + r);
+      if (gk + 1 < ke) b = *reinterpret_cast<const uint4 *>(src + (int64_t)(gk + 1) * sk + r);
+    }
+    const uint32_t aw[4] = {a.x, a.y, a.z, a.w}, bw[4] = {b.x, b.y, b.z, b.w};
+    uint32_t p[8];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      p[2 * q] = __byte_perm(aw[q], bw[q], 0x5410);
+      p[2 * q + 1] = __byte_perm(aw[q], bw[q], 0x7632);
+    }
+    unsigned char *d = dst + tc_off(r, k);
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      const int x = (q + rg) & 7;
+      uint32_t v = p[0];
+#pragma unroll
+      for (int z = 1; z < 8; ++z) v = x == z ? p[z] : v;
+      *reinterpret_cast<uint32_t *>(d + 16 * x) = v;
+    }
+  }
+}
+
 // Split K: CTA z sums K in [z kchunk, min(K, (z + 1) kchunk)) and writes its
 // partial tile to C + z cz (the caller reduces the partials).
 // tma: bit 0 loads A, bit 1 loads B through the tensor maps (rows x K, K
@@ -173,6 +210,10 @@ __global__ void __launch_bounds__(TC_THREADS) k_gemm_tc(int M, int N, int K,
   const bool a_vec = a_k1 && sam % 8 == 0 && (reinterpret_cast<uintptr_t>(A) & 15) == 0;
   const bool b_vec = b_k1 && sbn % 8 == 0 && (reinterpret_cast<uintptr_t>(B) & 15) == 0;
   const bool a_kfast = sak <= sam, b_kfast = sbk <= sbn;
+  // M- or N-contiguous operands (the weight gradients): 16-byte loads of
+  // eight rows, transposed on the way into shared memory
+  const bool a_m1 = sam == 1 && sak % 8 == 0 && M % 8 == 0 && (reinterpret_cast<uintptr_t>(A) & 15) == 0;
+  const bool b_n1 = sbn == 1 && sbk % 8 == 0 && N % 8 == 0 && (reinterpret_cast<uintptr_t>(B) & 15) == 0;
   uint32_t phase = 0, fphase = 0;
   bool ok = true, tma_pending = false;
   const int nk = (ke - kb + TC_BK - 1) / TC_BK;
@@ -207,6 +248,8 @@ __global__ void __launch_bounds__(TC_THREADS) k_gemm_tc(int M, int N, int K,
         tc_stage_row(sA + tc_off(r, kc), A + (int64_t)(gm < M ? gm : 0) * sam, 1, a_vec,
                      gm < M, k0 + kc, ke);
       }
+    } else if (a_m1) {
+      tc_stage_t(sA, A + m0, sak, M - m0, k0, ke);
     } else {
       for (int e = tid; e < TC_BM * TC_BK; e += TC_THREADS) {
         const int r = a_kfast ? e / TC_BK : e % TC_BM, k = a_kfast ? e % TC_BK : e / TC_BM;
@@ -223,6 +266,8 @@ __global__ void __launch_bounds__(TC_THREADS) k_gemm_tc(int M, int N, int K,
         tc_stage_row(sB + tc_off(c, kc), B + (int64_t)(gn < N ? gn : 0) * sbn, 1, b_vec,
                      gn < N, k0 + kc, ke);
       }
+    } else if (b_n1) {
+      tc_stage_t(sB, B + n0, sbk, N - n0, k0, ke);
     } else {
       for (int e = tid; e < TC_BN * TC_BK; e += TC_THREADS) {
         const int c = b_kfast ? e / TC_BK : e % TC_BN, k = b_kfast ? e % TC_BK : e / TC_BN;
@@ -299,6 +344,249 @@ __global__ void __launch_bounds__(TC_THREADS) k_gemm_tc(int M, int N, int K,
     if (tid == 0) atomicOr(err, 1);
     if (tma_pending) (void)tc_wait(mf, fphase);  // boxes still landing
     else (void)tc_wait(mb, phase ^ 1u);          // the last commit, if it is still pending
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  if (warp == 0)
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem),
+                 "r"(TC_TMEM_COLS)
+                 : "memory");
+}
+
+// ---------------------------------------------------------------------------
+// The same GEMM for two K-contiguous operands with what follows it fused into
+// the epilogue (the forward pass and the input gradients).  What bounded
+// k_gemm_tc here were its loads: boxes of 16-byte rows (2048 TMA requests per
+// slice) and no overlap of loads and MMAs, 1.7 to 3.1 % of the tensor pipe.
+// Here a slice is one 128-byte-row box per operand in the 128-byte swizzle
+// (rows of 64 K, 8-row groups 1024 bytes apart), three slices are in flight on
+// full / empty mbarriers, and bias, SiLU, its derivative, the loss gradient or
+// the prediction's de-standardisation run on the accumulator as it leaves
+// tensor memory, so no FP32 product is written and read back.  The MMAs and
+// their K order are k_gemm_tc's: the same bits.
+// ---------------------------------------------------------------------------
+constexpr int KK_STAGES = 3;
+constexpr int KK_STAGE_BYTES = 2 * TC_BM * TC_BK * 2;
+constexpr size_t KK_SMEM = (size_t)KK_STAGES * KK_STAGE_BYTES + 1024;  // two CTAs per SM
+
+enum { EP_HIDDEN = 0, EP_OUT, EP_MSE, EP_BACK, EP_UNPACK };
+
+struct Epilogue {
+  int mode;
+  const float *bias;       // forward modes
+  float *a;                // HIDDEN: pre-activation out (or null); BACK: in
+  __nv_bfloat16 *hb;       // HIDDEN: activation
+  float *out;              // OUT: [M][dout]
+  int dout;
+  const float *tgt;        // MSE: targets [.][dout], gathered through rows when given
+  const int32_t *rows;
+  int64_t nrows;
+  float *g;                // MSE, BACK: gradient, FP32 and BF16
+  __nv_bfloat16 *gb;
+  float *loss;
+  const float *mean, *stdv;  // UNPACK
+  double dt, *h0, *z0;
+};
+
+// exact float -> double on the integer pipe (the conversion unit shares the
+// FP64 pipe's rate); zeros kept, subnormals and non-finite values converted
+__device__ __forceinline__ double widen(float v) {
+  const unsigned u = __float_as_uint(v), e = u & 0x7f800000u;
+  if (e == 0x7f800000u || (e == 0 && (u << 1) != 0)) return (double)v;
+  const unsigned hi = (u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + (e ? 0x38000000u : 0u));
+  return __hiloint2double((int)hi, (int)(u << 29));
+}
+
+// sixteen accumulators of row r, columns c0 .. c0 + 15 (n of them inside)
+__device__ __forceinline__ void kk_epilogue(const Epilogue &ep, int64_t M, int N, int64_t r, int c0,
+                                            int n, const uint32_t (&v)[16], float &loss) {
+  const int64_t o = r * N + c0;
+  if (ep.mode == EP_HIDDEN || ep.mode == EP_BACK) {
+    __align__(16) float x[16];
+    __align__(16) __nv_bfloat16 b[16];
+    const bool back = ep.mode == EP_BACK;
+#pragma unroll
+    for (int q = 0; q < 4; ++q)  // N is a multiple of 8: n is 8 or 16
+      if (4 * q < n) {
+        const float4 in = back ? *reinterpret_cast<const float4 *>(ep.a + o + 4 * q)
+                               : *reinterpret_cast<const float4 *>(ep.bias + c0 + 4 * q);
+        const float p[4] = {in.x, in.y, in.z, in.w};
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+          const float acc = __uint_as_float(v[4 * q + t]);
+          x[4 * q + t] = back ? acc * silu_grad(p[t]) : acc + p[t];
+          b[4 * q + t] = __float2bfloat16(back ? x[4 * q + t] : silu(x[4 * q + t]));
+        }
+      }
+    float *f = back ? ep.g : ep.a;
+    __nv_bfloat16 *h = back ? ep.gb : ep.hb;
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      if (f && 4 * q < n)
+        *reinterpret_cast<float4 *>(f + o + 4 * q) = *reinterpret_cast<const float4 *>(x + 4 * q);
+#pragma unroll
+    for (int q = 0; q < 2; ++q)
+      if (8 * q < n)
+        *reinterpret_cast<uint4 *>(h + o + 8 * q) = *reinterpret_cast<const uint4 *>(b + 8 * q);
+    return;
+  }
+  int64_t tr = r;
+  if (ep.mode == EP_MSE && ep.rows) {
+    const int32_t s = ep.rows[r];
+    tr = (s >= 0 && (int64_t)s < ep.nrows) ? (int64_t)s : -1;
+  }
+  const float scale = (float)(M * ep.dout);
+#pragma unroll
+  for (int j = 0; j < 16; ++j) {
+    const int c = c0 + j;
+    if (j >= n) break;
+    const float y = __uint_as_float(v[j]) + ep.bias[c];
+    if (ep.mode == EP_OUT) {
+      if (c < ep.dout) ep.out[r * ep.dout + c] = y;
+    } else if (ep.mode == EP_MSE) {
+      float g = 0.0f;
+      if (c < ep.dout) {
+        const float d = y - (tr >= 0 ? ep.tgt[tr * ep.dout + c] : 0.0f);
+        g = 2.0f * d / scale;
+        loss += d * d / scale;
+      }
+      ep.g[o + j] = g;
+      ep.gb[o + j] = __float2bfloat16(g);
+    } else if (c < ep.dout) {
+      const double sd = widen(ep.stdv[c]), mu = widen(ep.mean[c]);
+      if (c == 0) {
+        if (ep.h0) ep.h0[r] = fmin(fmax(exp(widen(y) * sd + mu), 1e-14), ep.dt);
+      } else if (ep.z0) {
+        ep.z0[(int64_t)(c - 1) * M + r] = widen(y) * sd + mu;
+      }
+    }
+  }
+}
+
+__device__ __forceinline__ void tma_box(uint32_t dst, const CUtensorMap *tm, int x, int y,
+                                        uint32_t mbar) {
+  asm volatile(
+      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes"
+      " [%0], [%1, {%2, %3}], [%4];" ::"r"(dst),
+      "l"(reinterpret_cast<uint64_t>(tm)), "r"(x), "r"(y), "r"(mbar)
+      : "memory");
+}
+
+__global__ void __launch_bounds__(TC_THREADS) k_gemm_kk(int64_t M, int N, int K, int *err,
+                                                       const __grid_constant__ CUtensorMap tmA,
+                                                       const __grid_constant__ CUtensorMap tmB,
+                                                       const __grid_constant__ Epilogue ep) {
+  extern __shared__ unsigned char kk_raw[];
+  __shared__ __align__(8) unsigned long long full[KK_STAGES], empty[KK_STAGES], alldone;
+  __shared__ uint32_t tmem_base;
+  __shared__ int failed;
+  const uint32_t base = (smem_u32(kk_raw) + 1023u) & ~1023u;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int64_t m0 = (int64_t)blockIdx.x * TC_BM;
+  const int n0 = blockIdx.y * TC_BN;
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                     smem_u32(&tmem_base)),
+                 "r"(TC_TMEM_COLS)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  if (tid == 0) {
+    failed = 0;
+    for (int s = 0; s < KK_STAGES; ++s) {
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&full[s])) : "memory");
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&empty[s])) : "memory");
+    }
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&alldone)) : "memory");
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t tmem = tmem_base;
+  const int nk = (K + TC_BK - 1) / TC_BK;
+  if (tid == 0) {
+    auto load = [&](int kt) {
+      const int s = kt % KK_STAGES;
+      const uint32_t mb = smem_u32(&full[s]), dst = base + (uint32_t)(s * KK_STAGE_BYTES);
+      asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(mb),
+                   "r"((uint32_t)KK_STAGE_BYTES)
+                   : "memory");
+      // x = 64 kt: a multiple of 8 elements (16 bytes); zero fill past the matrix
+      tma_box(dst, &tmA, kt * TC_BK, (int)m0, mb);
+      tma_box(dst + KK_STAGE_BYTES / 2, &tmB, kt * TC_BK, n0, mb);
+    };
+    int loaded = 0;
+    for (; loaded < nk && loaded < KK_STAGES; ++loaded) load(loaded);
+    bool ok = true;
+    int kt = 0;
+    for (; kt < nk && ok; ++kt) {
+      const int s = kt % KK_STAGES;
+      const uint32_t ph = (uint32_t)(kt / KK_STAGES) & 1u;
+      ok = tc_wait(smem_u32(&full[s]), ph);
+      if (!ok) break;
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      const uint32_t sa = base + (uint32_t)(s * KK_STAGE_BYTES), sb = sa + KK_STAGE_BYTES / 2;
+#pragma unroll
+      for (int q = 0; q < TC_BK / 16; ++q) {
+        // 128-byte swizzle (layout 2): K advances by 32 bytes inside the row
+        const uint64_t sw = (uint64_t)2 << 61;
+        const uint64_t da = tc_desc(sa + 32u * q, 16u, 1024u) | sw;
+        const uint64_t db = tc_desc(sb + 32u * q, 16u, 1024u) | sw;
+        const uint32_t acc = (kt > 0 || q > 0) ? 1u : 0u;
+        asm volatile(
+            "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+            " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem),
+            "l"(da), "l"(db), "r"(tc_idesc(TC_BM, TC_BN)), "r"(acc)
+            : "memory");
+      }
+      asm volatile(
+          "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+              smem_u32(&empty[s]))
+          : "memory");
+      if (loaded < nk) {  // the stage is free once its MMAs are done
+        ok = tc_wait(smem_u32(&empty[s]), ph);
+        if (ok) load(loaded++);
+      }
+    }
+    asm volatile(
+        "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+            smem_u32(&alldone))
+        : "memory");
+    if (!ok) {  // flagged; wait (bounded) for the boxes still in flight
+      failed = 1;
+      atomicOr(err, 1);
+      for (int q = kt; q < loaded; ++q)
+        (void)tc_wait(smem_u32(&full[q % KK_STAGES]), (uint32_t)(q / KK_STAGES) & 1u);
+    }
+  }
+  __syncwarp();
+  const bool done = tc_wait(smem_u32(&alldone), 0);
+  if (!done) atomicOr(err, 1);
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const bool good = __syncthreads_and(done) && !failed;
+  float loss = 0.0f;
+  if (good) {
+    const int64_t row = m0 + warp * 32 + lane;
+    const int nc = N - n0 < TC_BN ? N - n0 : TC_BN;
+    for (int c0 = 0; c0 < nc; c0 += 16) {
+      uint32_t v[16];
+      const uint32_t taddr = tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0;
+      asm volatile(
+          "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,"
+          "%14,%15}, [%16];\n"
+          : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]),
+            "=r"(v[7]), "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]),
+            "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
+          : "r"(taddr)
+          : "memory");
+      asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+      if (row < M) kk_epilogue(ep, M, N, row, n0 + c0, min(16, nc - c0), v, loss);
+    }
+    if (ep.mode == EP_MSE) {
+      for (int o = 16; o > 0; o >>= 1) loss += __shfl_down_sync(0xffffffffu, loss, o);
+      if (lane == 0 && loss != 0.0f) atomicAdd(ep.loss, loss);
+    }
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
@@ -393,27 +681,73 @@ __global__ void k_silu_back(int64_t n, const float *dH, const float *a, float *g
   if (gb) gb[i] = __float2bfloat16(v);
 }
 
-// column sums: out[c] = sum_r g[r][c]
-__global__ void k_colsum(int64_t M, int N, const float *g, float *out) {
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= N) return;
+// column sums: out[c] = sum_r g[r][c]; a block per 32 columns, 32 row lanes
+// (a thread per column alone walked 4096 rows in sequence: 300 us)
+__global__ void __launch_bounds__(1024) k_colsum(int64_t M, int N, const float *g, float *out) {
+  __shared__ float part[32][33];
+  const int c = blockIdx.x * 32 + (threadIdx.x & 31), y = threadIdx.x >> 5;
   float s = 0.0f;
-  for (int64_t r = 0; r < M; ++r) s += g[r * N + c];
-  out[c] = s;
+  if (c < N) {
+#pragma unroll 4
+    for (int64_t r = y; r < M; r += 32) s += g[r * N + c];
+  }
+  part[y][threadIdx.x & 31] = s;
+  __syncthreads();
+  float t = part[threadIdx.x & 31][y];
+  for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+  const int co = blockIdx.x * 32 + y;
+  if ((threadIdx.x & 31) == 0 && co < N) out[co] = t;
 }
 
-// Adam with bias correction on the masked parameters
-__global__ void k_adam(int64_t n, float *p, const float *grad, float *m, float *v,
-                       const unsigned char *mask, float lr, float b1, float b2, float eps,
-                       float c1, float c2) {
+// weight blocks of the network: offset, K, N per layer
+struct LayerShapes {
+  int64_t woff[4];
+  int K[4], N[4];
+};
+
+// Adam, then the BF16 copies of the weight (as it lies and transposed)
+__global__ void k_adam_refresh(int64_t n, float *p, const float *grad, float *m, float *v,
+                               const unsigned char *mask, float lr, float b1, float b2, float eps,
+                               float c1, float c2, LayerShapes L, __nv_bfloat16 *wb,
+                               __nv_bfloat16 *wbt) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n || !mask[i]) return;
-  const float gi = grad[i];
-  const float mi = b1 * m[i] + (1.0f - b1) * gi;
-  const float vi = b2 * v[i] + (1.0f - b2) * gi * gi;
-  m[i] = mi;
-  v[i] = vi;
-  p[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+  if (i >= n) return;
+  float pi = p[i];
+  if (mask[i]) {
+    const float gi = grad[i];
+    const float mi = b1 * m[i] + (1.0f - b1) * gi;
+    const float vi = b2 * v[i] + (1.0f - b2) * gi * gi;
+    m[i] = mi;
+    v[i] = vi;
+    pi -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+    p[i] = pi;
+  }
+  const __nv_bfloat16 b = __float2bfloat16(pi);
+  wb[i] = b;
+#pragma unroll
+  for (int l = 0; l < 4; ++l) {
+    const int64_t e = i - L.woff[l];
+    if (e >= 0 && e < (int64_t)L.K[l] * L.N[l]) {
+      const int k = (int)(e / L.N[l]), c = (int)(e % L.N[l]);
+      wbt[L.woff[l] + (int64_t)c * L.K[l] + k] = b;
+    }
+  }
+}
+
+// input rows [M][din] (gathered through rows when given; an index outside
+// [0, R) gives a zero row) -> BF16 [M][ld], zero padded
+__global__ void k_gather_pack(int64_t M, int din, int ld, const float *X, int64_t R,
+                              const int32_t *rows, __nv_bfloat16 *xb) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= M * ld) return;
+  const int64_t r = i / ld;
+  const int c = (int)(i % ld);
+  int64_t s = r;
+  if (rows) {
+    const int32_t q = rows[r];
+    s = (q >= 0 && (int64_t)q < R) ? (int64_t)q : -1;
+  }
+  xb[i] = __float2bfloat16(s >= 0 && c < din ? X[s * din + c] : 0.0f);
 }
 
 __global__ void k_to_bf16(int64_t n, const float *x, __nv_bfloat16 *y) {
@@ -443,35 +777,158 @@ __global__ void k_splitk_reduce(int M, int N, int S, const float *ws, float *C, 
   *dst = accumulate ? *dst + v : v;
 }
 
-// column mean and standard deviation of X [M][d] (two-pass, FP64 sums)
-__global__ void k_moments(int64_t M, int d, const float *X, float *mean, float *stdv) {
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= d) return;
-  double s = 0.0;
-  for (int64_t r = 0; r < M; ++r) s += X[r * d + c];
-  const double mu = s / (double)M;
-  double q = 0.0;
-  for (int64_t r = 0; r < M; ++r) {
-    const double e = X[r * d + c] - mu;
-    q += e * e;
+// column mean and standard deviation of X [M][d] (two-pass, FP64 sums).  A
+// cluster of eight CTAs owns eight columns (one 32-byte sector per row) and
+// sums them through distributed shared memory: two passes in one launch
+// without a workspace.  Bound by FP64 additions; a thread per column walked
+// the rows in sequence (65536 x 160: 14 ms).  The FP32 values are widened on
+// the integer pipe.
+constexpr int MOM_CTAS = 8, MOM_COLS = 8, MOM_THREADS = 512;
+
+__global__ void __cluster_dims__(MOM_CTAS, 1, 1) __launch_bounds__(MOM_THREADS)
+    k_moments(int64_t M, int d, const float *X, float *mean, float *stdv) {
+  namespace cg = cooperative_groups;
+  cg::cluster_group cl = cg::this_cluster();
+  __shared__ double part[2][MOM_COLS];  // this CTA's sums, per pass
+  __shared__ double warp_part[MOM_THREADS / 32][MOM_COLS];
+  const int tid = threadIdx.x, cx = tid % MOM_COLS, warp = tid / 32;
+  const int c = (int)(blockIdx.x / MOM_CTAS) * MOM_COLS + cx;
+  const int64_t step = (int64_t)MOM_CTAS * (MOM_THREADS / MOM_COLS);
+  const int64_t r0 = (int64_t)cl.block_rank() * (MOM_THREADS / MOM_COLS) + tid / MOM_COLS;
+  double mu = 0.0, q = 0.0;
+  for (int pass = 0; pass < 2; ++pass) {
+    double s = 0.0;
+    if (c < d) {
+      int64_t r = r0;
+      for (; r + 3 * step < M; r += 4 * step) {  // four rows' loads in flight
+        const float a0 = X[r * d + c], a1 = X[(r + step) * d + c], a2 = X[(r + 2 * step) * d + c],
+                    a3 = X[(r + 3 * step) * d + c];
+        if (pass == 0) {
+          s += (widen(a0) + widen(a1)) + (widen(a2) + widen(a3));
+        } else {
+          const double e0 = widen(a0) - mu, e1 = widen(a1) - mu, e2 = widen(a2) - mu,
+                       e3 = widen(a3) - mu;
+          s = fma(e0, e0, fma(e1, e1, fma(e2, e2, fma(e3, e3, s))));
+        }
+      }
+      for (; r < M; r += step) {
+        const double e = widen(X[r * d + c]) - mu;
+        s += pass == 0 ? e : e * e;
+      }
+    }
+    for (int o = 16; o >= MOM_COLS; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if ((tid & 31) < MOM_COLS) warp_part[warp][cx] = s;
+    __syncthreads();
+    if (tid < MOM_COLS) {
+      double t = 0.0;
+      for (int w = 0; w < MOM_THREADS / 32; ++w) t += warp_part[w][tid];
+      part[pass][tid] = t;
+    }
+    cl.sync();
+    double t = 0.0;
+    for (int k = 0; k < MOM_CTAS; ++k) t += cl.map_shared_rank(&part[pass][0], k)[cx];
+    if (pass == 0)
+      mu = t / (double)M;
+    else
+      q = t;
   }
-  mean[c] = (float)mu;
-  stdv[c] = (float)fmax(sqrt(q / (double)M), 1e-12);
+  if (c < d && cl.block_rank() == 0 && tid < MOM_COLS) {
+    mean[c] = (float)mu;
+    stdv[c] = (float)fmax(sqrt(q / (double)M), 1e-12);
+  }
+  cl.sync();  // the peers' sums stay readable until all are done
 }
 
-// features of the integrator's states: [log T, log P, log dt, log10 Y_k], standardised
-__global__ void k_features(int64_t n, int ns, const double *Y, const double *T, const double *P,
-                           double dt, const float *mean, const float *stdv, float *X) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const int din = 3 + ns;
-  float *x = X + i * din;
-  x[0] = (float)log(T[i]);
-  x[1] = (float)log(P[i]);
-  x[2] = (float)log(dt);
-  for (int k = 0; k < ns; ++k) x[3 + k] = (float)log10(fmax(Y[(int64_t)k * n + i], 1e-12));
-  if (mean)
-    for (int c = 0; c < din; ++c) x[c] = (x[c] - mean[c]) / stdv[c];
+// ---------------------------------------------------------------------------
+// Natural logarithm by table (Tang, ACM TOMS 16, 1990): x = 2^e m, an entry
+// c near 1/m for each 1/128 of [1, 2), r = m c - 1 (|r| < 2^-7), log x = e ln2
+// - log c + log1p(r), the last by its series to r^8 (2^-59 of r).  A dozen FP64
+// operations against the library's 35; normal positive x only.
+// tab[2 j] = c, tab[2 j + 1] = -log c; a block fills its own copy.
+// ---------------------------------------------------------------------------
+constexpr int LOG_TAB = 128;
+
+__device__ __forceinline__ void log_table(double *tab) {
+  for (int j = threadIdx.x; j < LOG_TAB; j += blockDim.x) {
+    // nine significant bits, so m c has no more than 62 and r one rounding
+    // (1 and 1/2 at the ends keep log x accurate relative to itself near 1)
+    const int q = j == 0 ? 512 : j == LOG_TAB - 1 ? 256 : __float2int_rn(65536.0f / (128.5f + j));
+    const double c = q / 512.0;
+    tab[2 * j] = c;
+    tab[2 * j + 1] = -log(c);
+  }
+}
+
+__device__ __forceinline__ double tab_log(double x, const double *tab) {
+  const long long b = __double_as_longlong(x);
+  const int hi = (int)(b >> 32);
+  if ((unsigned)(hi - 0x00100000) >= 0x7fe00000u) return log(x);  // 0, < 0, subnormal, inf, NaN
+  const int j = (hi >> 13) & (LOG_TAB - 1), e = (hi >> 20) - 1023;
+  const double m = __longlong_as_double((b & 0x000fffffffffffffll) | 0x3ff0000000000000ll);
+  const double r = fma(m, tab[2 * j], -1.0);
+  // e as a double without the conversion unit: 2^52 + 2^51 + e, less that
+  const double ed = __longlong_as_double(0x4338000000000000ll + e) - 6755399441055744.0;
+  double p = fma(r, -1.0 / 8.0, 1.0 / 7.0);
+  p = fma(p, r, -1.0 / 6.0);
+  p = fma(p, r, 1.0 / 5.0);
+  p = fma(p, r, -1.0 / 4.0);
+  p = fma(p, r, 1.0 / 3.0);
+  p = fma(p, r, -0.5);
+  p = fma(p * r, r, r);
+  return fma(ed, 0.693147180559945309417, tab[2 * j + 1] + p);
+}
+
+// features of the integrator's states: [log T, log P, log dt, log10 Y_k],
+// standardised with mean / stdv when given, as FP32 rows X [n][3 + ns] or as
+// BF16 rows xb [n][ld] with zero padding.  A block stages FEAT_ROWS states in
+// shared memory: the species-major reads and the row-major writes are both
+// coalesced.  Bound by the FP64 work of the logarithms.
+constexpr int FEAT_ROWS = 32, FEAT_COLS = 256, FEAT_THREADS = 256;
+
+__global__ void __launch_bounds__(FEAT_THREADS)
+    k_features(int64_t n, int ns, const double *Y, const double *T, const double *P, double logdt,
+               const float *mean, const float *stdv, float *X, __nv_bfloat16 *xb, int ld) {
+  __shared__ double tab[2 * LOG_TAB];
+  __shared__ float tile[FEAT_ROWS][FEAT_COLS + 1];
+  const int din = 3 + ns, tid = threadIdx.x;
+  log_table(tab);
+  __syncthreads();
+  for (int64_t i0 = (int64_t)blockIdx.x * FEAT_ROWS; i0 < n; i0 += (int64_t)gridDim.x * FEAT_ROWS) {
+    const int rows = (int)(n - i0 < FEAT_ROWS ? n - i0 : FEAT_ROWS);
+    for (int c0 = 0; c0 < din; c0 += FEAT_COLS) {
+      const int nc = din - c0 < FEAT_COLS ? din - c0 : FEAT_COLS;
+      for (int q = tid; q < FEAT_ROWS * nc; q += FEAT_THREADS) {
+        const int row = q % FEAT_ROWS, c = c0 + q / FEAT_ROWS;
+        const int64_t i = i0 + row;
+        if (row >= rows) continue;
+        float x;
+        if (c == 2) {
+          x = (float)logdt;
+        } else if (c < 2) {
+          x = (float)tab_log((c == 0 ? T : P)[i], tab);
+        } else {
+          const double y = Y[(int64_t)(c - 3) * n + i];
+          // max(y, 1e-12) on the bit pattern: negative values and NaN give the floor
+          const long long yb = __double_as_longlong(y), fl = __double_as_longlong(1e-12);
+          const double z = (yb > fl && yb <= 0x7ff0000000000000ll) ? y : 1e-12;
+          x = (float)(tab_log(z, tab) * 0.434294481903251827651);
+        }
+        if (mean) x = (x - mean[c]) / stdv[c];
+        tile[row][c - c0] = x;
+      }
+      __syncthreads();
+      if (X)
+        for (int q = tid; q < rows * nc; q += FEAT_THREADS)
+          X[(i0 + q / nc) * din + c0 + q % nc] = tile[q / nc][q % nc];
+      if (xb)
+        for (int q = tid; q < rows * nc; q += FEAT_THREADS)
+          xb[(i0 + q / nc) * ld + c0 + q % nc] = __float2bfloat16(tile[q / nc][q % nc]);
+      __syncthreads();
+    }
+    if (xb)
+      for (int q = tid; q < rows * (ld - din); q += FEAT_THREADS)
+        xb[(i0 + q / (ld - din)) * ld + din + q % (ld - din)] = __float2bfloat16(0.0f);
+  }
 }
 
 // network outputs -> h0 (clipped to [1e-14, dt]) and stage guesses [3N][n]
@@ -489,20 +946,31 @@ __global__ void k_unpack_prediction(int64_t n, int dout, int ld, const float *y,
     for (int c = 1; c < dout; ++c) z0[(int64_t)(c - 1) * n + i] = (double)r[c] * stdv[c] + mean[c];
 }
 
-// training targets: [log h, z_1..z_3N] from the integrator's first-step outputs
-__global__ void k_targets(int64_t n, int nz, const double *h, const double *z, float *tgt) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  float *t = tgt + i * (1 + nz);
-  t[0] = (float)log(h[i]);
-  for (int c = 0; c < nz; ++c) t[1 + c] = (float)z[(int64_t)c * n + i];
-}
-
-__global__ void k_standardise(int64_t M, int d, float *X, const float *mean, const float *stdv) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= M * d) return;
-  const int c = (int)(i % d);
-  X[i] = (X[i] - mean[c]) / stdv[c];
+// training targets: [log h, z_1..z_3N] from the integrator's first-step
+// outputs, standardised when mean is given; staged like the features
+__global__ void __launch_bounds__(FEAT_THREADS)
+    k_targets(int64_t n, int nz, const double *h, const double *z, const float *mean,
+              const float *stdv, float *tgt) {
+  __shared__ float tile[FEAT_ROWS][FEAT_COLS + 1];
+  const int d = 1 + nz, tid = threadIdx.x;
+  for (int64_t i0 = (int64_t)blockIdx.x * FEAT_ROWS; i0 < n; i0 += (int64_t)gridDim.x * FEAT_ROWS) {
+    const int rows = (int)(n - i0 < FEAT_ROWS ? n - i0 : FEAT_ROWS);
+    for (int c0 = 0; c0 < d; c0 += FEAT_COLS) {
+      const int nc = d - c0 < FEAT_COLS ? d - c0 : FEAT_COLS;
+      for (int q = tid; q < FEAT_ROWS * nc; q += FEAT_THREADS) {
+        const int row = q % FEAT_ROWS, c = c0 + q / FEAT_ROWS;
+        const int64_t i = i0 + row;
+        if (row >= rows) continue;
+        float x = c == 0 ? (float)log(h[i]) : (float)z[(int64_t)(c - 1) * n + i];
+        if (mean) x = (x - mean[c]) / stdv[c];
+        tile[row][c - c0] = x;
+      }
+      __syncthreads();
+      for (int q = tid; q < rows * nc; q += FEAT_THREADS)
+        tgt[(i0 + q / nc) * d + c0 + q % nc] = tile[q / nc][q % nc];
+      __syncthreads();
+    }
+  }
 }
 
 inline unsigned blocks(int64_t n, int b = 256) { return (unsigned)((n + b - 1) / b); }
@@ -526,7 +994,7 @@ struct kin_mlp {
         *dH = nullptr, *y = nullptr, *loss = nullptr;
   float *xg = nullptr, *tg = nullptr;  // gathered minibatch rows (train_step_rows)
   int *err = nullptr;                  // set by a tensor-core GEMM whose wait expired
-  __nv_bfloat16 *xb = nullptr, *hb[LAYERS] = {}, *gb = nullptr;
+  __nv_bfloat16 *xb = nullptr, *hb[LAYERS] = {}, *gb = nullptr, *gb2 = nullptr;
 };
 
 static int mlp_reserve(kin_mlp *n, int64_t rows) {
@@ -540,6 +1008,7 @@ static int mlp_reserve(kin_mlp *n, int64_t rows) {
   cudaFree(n->g);
   cudaFree(n->dH);
   cudaFree(n->gb);
+  cudaFree(n->gb2);
   for (int l = 0; l < LAYERS; ++l) {
     cudaFree(n->a[l]);
     cudaFree(n->hf[l]);
@@ -555,6 +1024,7 @@ static int mlp_reserve(kin_mlp *n, int64_t rows) {
   KIN_CUDA_TRY(cudaMalloc(&n->g, sizeof(float) * rows * wmax));
   KIN_CUDA_TRY(cudaMalloc(&n->dH, sizeof(float) * rows * wmax));
   KIN_CUDA_TRY(cudaMalloc(&n->gb, sizeof(__nv_bfloat16) * rows * wmax));
+  KIN_CUDA_TRY(cudaMalloc(&n->gb2, sizeof(__nv_bfloat16) * rows * wmax));
   for (int l = 0; l < LAYERS; ++l) {
     KIN_CUDA_TRY(cudaMalloc(&n->a[l], sizeof(float) * rows * n->N[l]));
     KIN_CUDA_TRY(cudaMalloc(&n->hf[l], sizeof(float) * rows * n->N[l]));
@@ -582,9 +1052,11 @@ static PFN_cuTensorMapEncodeTiled_v12000 tmap_encoder() {
 }
 
 // tensor map of a rows x cols BF16 matrix with row stride ld (elements),
-// boxes of 8 columns x 128 rows, zero fill outside; false when the layout
+// boxes of 8 columns x 128 rows (swizzle: 64 columns in the 128-byte swizzle),
+// zero fill outside; false when the layout
 // does not allow the TMA (16-byte base and rows)
-static bool make_tmap(CUtensorMap *m, const void *base, int64_t rows, int64_t cols, int64_t ld) {
+static bool make_tmap(CUtensorMap *m, const void *base, int64_t rows, int64_t cols, int64_t ld,
+                      bool swizzle = false) {
   std::memset(m, 0, sizeof *m);
   auto enc = tmap_encoder();
   if (!enc || (reinterpret_cast<uintptr_t>(base) & 15) || (ld * 2) % 16 || ld < cols ||
@@ -592,9 +1064,10 @@ static bool make_tmap(CUtensorMap *m, const void *base, int64_t rows, int64_t co
     return false;
   const cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
   const cuuint64_t strides[1] = {(cuuint64_t)ld * 2};
-  const cuuint32_t box[2] = {8, 128}, es[2] = {1, 1};
+  const cuuint32_t box[2] = {swizzle ? 64u : 8u, 128}, es[2] = {1, 1};
   return enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(base), dims, strides, box,
-             es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
+             es, CU_TENSOR_MAP_INTERLEAVE_NONE,
+             swizzle ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE,
              CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) ==
          CUDA_SUCCESS;
 }
@@ -644,6 +1117,79 @@ static void gemm(const kin_mlp *n, cudaStream_t st, int M, int N, int K, bool bf
   }
 }
 
+// The fused path: BF16, both operands of the forward and input-gradient GEMMs
+// in 16-byte rows.  Other widths keep the unfused kernels.
+static bool mlp_fused(const kin_mlp *n) {
+  return n->precision == 0 && n->width % 8 == 0 && tmap_encoder() != nullptr;
+}
+
+static int gemm_kk(const kin_mlp *n, cudaStream_t st, int64_t M, int N, int K,
+                   const __nv_bfloat16 *A, const __nv_bfloat16 *B, const Epilogue &ep) {
+  CUtensorMap tmA, tmB;
+  if (!make_tmap(&tmA, A, M, K, K, true) || !make_tmap(&tmB, B, N, K, K, true)) return KIN_ERR_CUDA;
+  const dim3 grid((unsigned)((M + TC_BM - 1) / TC_BM), (unsigned)((N + TC_BN - 1) / TC_BN), 1);
+  k_gemm_kk<<<grid, TC_THREADS, KK_SMEM, st>>>(M, N, K, n->err, tmA, tmB, ep);
+  KIN_CUDA_TRY(cudaGetLastError());
+  return KIN_OK;
+}
+
+// forward pass of the rows in xb; `last` is the output layer's epilogue
+static int mlp_forward_fused(kin_mlp *n, int64_t M, cudaStream_t st, bool keep, Epilogue last) {
+  for (int l = 0; l < LAYERS; ++l) {
+    Epilogue ep{};
+    if (l == LAYERS - 1) {
+      ep = last;
+    } else {
+      ep.mode = EP_HIDDEN;
+      ep.a = keep ? n->a[l] : nullptr;  // the backward pass's SiLU derivative
+      ep.hb = n->hb[l];
+    }
+    ep.bias = n->p + n->boff[l];
+    ep.dout = n->dout;
+    const int rc = gemm_kk(n, st, M, n->N[l], n->K[l], l ? n->hb[l - 1] : n->xb,
+                           n->wbt + n->woff[l], ep);
+    if (rc) return rc;
+  }
+  return KIN_OK;
+}
+
+// loss and gradients of the rows in xb against targets gathered through rows
+static int mlp_grad_fused(kin_mlp *n, int64_t M, const float *T, const int32_t *rows, int64_t R,
+                          float *loss, cudaStream_t st) {
+  KIN_CUDA_TRY(cudaMemsetAsync(loss, 0, sizeof(float), st));
+  Epilogue ep{};
+  ep.mode = EP_MSE;
+  ep.tgt = T;
+  ep.rows = rows;
+  ep.nrows = R;
+  ep.g = n->g;
+  ep.gb = n->gb;
+  ep.loss = loss;
+  int rc = mlp_forward_fused(n, M, st, true, ep);
+  if (rc) return rc;
+  // the gradient alternates between two buffer pairs: a layer's input
+  // gradient is written while its own gradient is read
+  float *g = n->g, *g2 = n->dH;
+  __nv_bfloat16 *gb = n->gb, *gb2 = n->gb2;
+  for (int l = LAYERS - 1; l >= 0; --l) {
+    const int K = n->K[l], N = n->N[l];
+    gemm(n, st, K, N, (int)M, true, l ? n->hb[l - 1] : n->xb, 1, K, gb, N, 1,
+         n->grad + n->woff[l], N, 0);
+    k_colsum<<<blocks(N, 32), 1024, 0, st>>>(M, N, g, n->grad + n->boff[l]);
+    if (l == 0) break;
+    Epilogue e{};
+    e.mode = EP_BACK;
+    e.a = n->a[l - 1];
+    e.g = g2;
+    e.gb = gb2;
+    if ((rc = gemm_kk(n, st, M, K, N, gb, n->wb + n->woff[l], e))) return rc;
+    std::swap(g, g2);
+    std::swap(gb, gb2);
+  }
+  KIN_CUDA_TRY(cudaGetLastError());
+  return KIN_OK;
+}
+
 // forward pass over M rows already packed in xf/xb; leaves y = hf[L-1]
 static int mlp_forward_packed(kin_mlp *n, int64_t M, cudaStream_t st) {
   const bool bf = n->precision == 0;
@@ -674,7 +1220,7 @@ static int mlp_backward(kin_mlp *n, int64_t M, cudaStream_t st) {
     const void *gv = bf ? (const void *)n->gb : (const void *)n->g;
     // dW[i][o] = sum_b h[b][i] g[b][o]
     gemm(n, st, K, N, (int)M, bf, hin, 1, K, gv, N, 1, n->grad + n->woff[l], N, 0);
-    k_colsum<<<blocks(N, 128), 128, 0, st>>>(M, N, n->g, n->grad + n->boff[l]);
+    k_colsum<<<blocks(N, 32), 1024, 0, st>>>(M, N, n->g, n->grad + n->boff[l]);
     if (l == 0) break;
     // dH[b][i] = sum_o g[b][o] W[i][o]
     const void *W = bf ? (const void *)(n->wb + n->woff[l]) : (const void *)(n->p + n->woff[l]);
@@ -691,6 +1237,16 @@ static int mlp_pack(kin_mlp *n, const float *X, int64_t M, cudaStream_t st) {
   if (rc) return rc;
   k_pack_input<<<blocks(M * n->dinp), 256, 0, st>>>(M, n->din, n->dinp, X, n->xf,
                                                     n->precision == 0 ? n->xb : nullptr);
+  KIN_CUDA_TRY(cudaGetLastError());
+  return KIN_OK;
+}
+
+// the rows of X (through rows, when given) as the fused path's BF16 input
+static int mlp_gather(kin_mlp *n, const float *X, int64_t R, const int32_t *rows, int64_t M,
+                      cudaStream_t st) {
+  const int rc = mlp_reserve(n, M);
+  if (rc) return rc;
+  k_gather_pack<<<blocks(M * n->dinp), 256, 0, st>>>(M, n->din, n->dinp, X, R, rows, n->xb);
   KIN_CUDA_TRY(cudaGetLastError());
   return KIN_OK;
 }
@@ -769,6 +1325,8 @@ extern "C" int kin_mlp_create(int32_t din, int32_t width, int32_t dout, int32_t 
       cudaMemset(n->err, 0, sizeof(int)) != cudaSuccess ||
       cudaFuncSetAttribute(k_gemm_tc, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)TC_SMEM) != cudaSuccess ||
+      cudaFuncSetAttribute(k_gemm_kk, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           (int)KK_SMEM) != cudaSuccess ||
       mlp_refresh_bf16(n, nullptr) != KIN_OK || cudaDeviceSynchronize() != cudaSuccess) {
     (void)cudaGetLastError();
     kin_mlp_destroy(n);
@@ -798,6 +1356,7 @@ extern "C" void kin_mlp_destroy(kin_mlp *n) {
   cudaFree(n->g);
   cudaFree(n->dH);
   cudaFree(n->gb);
+  cudaFree(n->gb2);
   for (int l = 0; l < LAYERS; ++l) {
     cudaFree(n->a[l]);
     cudaFree(n->hf[l]);
@@ -859,10 +1418,46 @@ extern "C" int kin_mlp_forward(kin_mlp *n, const float *X, float *Y, int64_t M, 
   if (!n || M < 0 || (M > 0 && (!X || !Y))) return KIN_ERR_INVALID_ARG;
   if (M == 0) return KIN_OK;
   cudaStream_t st = (cudaStream_t)stream;
+  if (mlp_fused(n)) {
+    const int rc = mlp_gather(n, X, 0, nullptr, M, st);
+    if (rc) return rc;
+    Epilogue ep{};
+    ep.mode = EP_OUT;
+    ep.out = Y;
+    return mlp_forward_fused(n, M, st, false, ep);
+  }
   int rc = mlp_pack(n, X, M, st);
   if (rc || (rc = mlp_forward_packed(n, M, st))) return rc;
   KIN_CUDA_TRY(cudaMemcpy2DAsync(Y, sizeof(float) * n->dout, n->y, sizeof(float) * n->doutp,
                                  sizeof(float) * n->dout, M, cudaMemcpyDeviceToDevice, st));
+  return KIN_OK;
+}
+
+// loss and gradients (into n->grad) of M rows, gathered through rows [M] out
+// of R when given
+static int mlp_loss_and_grad(kin_mlp *n, const float *X, const float *T, int64_t R,
+                             const int32_t *rows, int64_t M, float *loss_out, cudaStream_t st) {
+  int rc;
+  if (mlp_fused(n)) {
+    if ((rc = mlp_gather(n, X, R, rows, M, st))) return rc;
+    return mlp_grad_fused(n, M, T, rows, R, loss_out ? loss_out : n->loss, st);
+  }
+  if (rows) {
+    if ((rc = mlp_reserve(n, M))) return rc;
+    k_gather_rows<<<blocks(M * n->din), 256, 0, st>>>(M, n->din, X, R, rows, n->xg);
+    k_gather_rows<<<blocks(M * n->dout), 256, 0, st>>>(M, n->dout, T, R, rows, n->tg);
+    KIN_CUDA_TRY(cudaGetLastError());
+    X = n->xg;
+    T = n->tg;
+  }
+  rc = mlp_pack(n, X, M, st);
+  if (rc || (rc = mlp_forward_packed(n, M, st))) return rc;
+  KIN_CUDA_TRY(cudaMemsetAsync(n->loss, 0, sizeof(float), st));
+  k_mse_grad<<<blocks(M * n->doutp), 256, 0, st>>>(M, n->dout, n->doutp, n->y, T, n->g,
+                                                   n->precision == 0 ? n->gb : nullptr, n->loss);
+  if ((rc = mlp_backward(n, M, st))) return rc;
+  if (loss_out)
+    KIN_CUDA_TRY(cudaMemcpyAsync(loss_out, n->loss, sizeof(float), cudaMemcpyDeviceToDevice, st));
   return KIN_OK;
 }
 
@@ -871,14 +1466,8 @@ extern "C" int kin_mlp_grad(kin_mlp *n, const float *X, const float *T, int64_t 
                             float *loss_out, void *stream) {
   if (!n || M < 1 || !X || !T) return KIN_ERR_INVALID_ARG;
   cudaStream_t st = (cudaStream_t)stream;
-  int rc = mlp_pack(n, X, M, st);
-  if (rc || (rc = mlp_forward_packed(n, M, st))) return rc;
-  KIN_CUDA_TRY(cudaMemsetAsync(n->loss, 0, sizeof(float), st));
-  k_mse_grad<<<blocks(M * n->doutp), 256, 0, st>>>(M, n->dout, n->doutp, n->y, T, n->g,
-                                                   n->precision == 0 ? n->gb : nullptr, n->loss);
-  if ((rc = mlp_backward(n, M, st))) return rc;
-  if (loss_out)
-    KIN_CUDA_TRY(cudaMemcpyAsync(loss_out, n->loss, sizeof(float), cudaMemcpyDeviceToDevice, st));
+  int rc = mlp_loss_and_grad(n, X, T, 0, nullptr, M, loss_out, st);
+  if (rc) return rc;
   if (grad_out) {
     // gather the unpadded layout on the host side of the stream
     KIN_CUDA_TRY(cudaStreamSynchronize(st));
@@ -899,26 +1488,29 @@ extern "C" int kin_mlp_grad(kin_mlp *n, const float *X, const float *T, int64_t 
   return KIN_OK;
 }
 
+static int mlp_adam(kin_mlp *n, float lr, cudaStream_t st) {
+  n->step++;
+  const float b1 = 0.9f, b2 = 0.999f;
+  const float c1 = 1.0f - std::pow(b1, (float)n->step), c2 = 1.0f - std::pow(b2, (float)n->step);
+  LayerShapes L;
+  for (int l = 0; l < LAYERS; ++l) {
+    L.woff[l] = n->woff[l];
+    L.K[l] = n->K[l];
+    L.N[l] = n->N[l];
+  }
+  k_adam_refresh<<<blocks(n->np), 256, 0, st>>>(n->np, n->p, n->grad, n->m, n->v, n->mask, lr, b1,
+                                                b2, 1e-8f, c1, c2, L, n->wb, n->wbt);
+  KIN_CUDA_TRY(cudaGetLastError());
+  return KIN_OK;
+}
+
 // one Adam step on a minibatch (X dev [M][din], T dev [M][dout]); loss_out dev scalar or NULL
 extern "C" int kin_mlp_train_step(kin_mlp *n, const float *X, const float *T, int64_t M, float lr,
                                   float *loss_out, void *stream) {
   if (!n || M < 1 || !X || !T || !(lr > 0.0f)) return KIN_ERR_INVALID_ARG;
   cudaStream_t st = (cudaStream_t)stream;
-  int rc = mlp_pack(n, X, M, st);
-  if (rc || (rc = mlp_forward_packed(n, M, st))) return rc;
-  KIN_CUDA_TRY(cudaMemsetAsync(n->loss, 0, sizeof(float), st));
-  k_mse_grad<<<blocks(M * n->doutp), 256, 0, st>>>(M, n->dout, n->doutp, n->y, T, n->g,
-                                                   n->precision == 0 ? n->gb : nullptr, n->loss);
-  if ((rc = mlp_backward(n, M, st))) return rc;
-  n->step++;
-  const float b1 = 0.9f, b2 = 0.999f;
-  const float c1 = 1.0f - std::pow(b1, (float)n->step), c2 = 1.0f - std::pow(b2, (float)n->step);
-  k_adam<<<blocks(n->np), 256, 0, st>>>(n->np, n->p, n->grad, n->m, n->v, n->mask, lr, b1, b2,
-                                        1e-8f, c1, c2);
-  if ((rc = mlp_refresh_bf16(n, st))) return rc;
-  if (loss_out)
-    KIN_CUDA_TRY(cudaMemcpyAsync(loss_out, n->loss, sizeof(float), cudaMemcpyDeviceToDevice, st));
-  return KIN_OK;
+  const int rc = mlp_loss_and_grad(n, X, T, 0, nullptr, M, loss_out, st);
+  return rc ? rc : mlp_adam(n, lr, st);
 }
 
 extern "C" int kin_mlp_train_step_rows(kin_mlp *n, const float *X, const float *T, int64_t R,
@@ -926,18 +1518,28 @@ extern "C" int kin_mlp_train_step_rows(kin_mlp *n, const float *X, const float *
                                        void *stream) {
   if (!n || M < 1 || R < 1 || !X || !T || !rows || !(lr > 0.0f)) return KIN_ERR_INVALID_ARG;
   cudaStream_t st = (cudaStream_t)stream;
-  int rc = mlp_reserve(n, M);
-  if (rc) return rc;
-  k_gather_rows<<<blocks(M * n->din), 256, 0, st>>>(M, n->din, X, R, rows, n->xg);
-  k_gather_rows<<<blocks(M * n->dout), 256, 0, st>>>(M, n->dout, T, R, rows, n->tg);
-  KIN_CUDA_TRY(cudaGetLastError());
-  return kin_mlp_train_step(n, n->xg, n->tg, M, lr, loss_out, stream);
+  const int rc = mlp_loss_and_grad(n, X, T, R, rows, M, loss_out, st);
+  return rc ? rc : mlp_adam(n, lr, st);
 }
 
 extern "C" int kin_moments(const float *X, int64_t M, int32_t d, float *mean, float *stdv,
                            void *stream) {
   if (!X || M < 1 || d < 1 || !mean || !stdv) return KIN_ERR_INVALID_ARG;
-  k_moments<<<blocks(d, 64), 64, 0, (cudaStream_t)stream>>>(M, d, X, mean, stdv);
+  k_moments<<<MOM_CTAS * blocks(d, MOM_COLS), MOM_THREADS, 0, (cudaStream_t)stream>>>(M, d, X, mean,
+                                                                                     stdv);
+  KIN_CUDA_TRY(cudaGetLastError());
+  return KIN_OK;
+}
+
+static unsigned row_blocks(int64_t n) {
+  return (unsigned)std::min<int64_t>((n + FEAT_ROWS - 1) / FEAT_ROWS, 152 * 8);
+}
+
+static int launch_features(int ns, const double *Y, const double *T, const double *P, int64_t n,
+                           double dt, const float *mean, const float *stdv, float *X,
+                           __nv_bfloat16 *xb, int ld, cudaStream_t st) {
+  k_features<<<row_blocks(n), FEAT_THREADS, 0, st>>>(n, ns, Y, T, P, std::log(dt), mean, stdv, X,
+                                                     xb, ld);
   KIN_CUDA_TRY(cudaGetLastError());
   return KIN_OK;
 }
@@ -949,9 +1551,7 @@ extern "C" int kin_mlp_features(int32_t ns, const double *Y, const double *T, co
       ((mean == nullptr) != (stdv == nullptr)))
     return KIN_ERR_INVALID_ARG;
   if (n == 0) return KIN_OK;
-  k_features<<<blocks(n), 256, 0, (cudaStream_t)stream>>>(n, ns, Y, T, P, dt, mean, stdv, X);
-  KIN_CUDA_TRY(cudaGetLastError());
-  return KIN_OK;
+  return launch_features(ns, Y, T, P, n, dt, mean, stdv, X, nullptr, 0, (cudaStream_t)stream);
 }
 
 extern "C" int kin_mlp_targets(int32_t nz, const double *h, const double *z, int64_t n,
@@ -959,8 +1559,7 @@ extern "C" int kin_mlp_targets(int32_t nz, const double *h, const double *z, int
   if (nz < 1 || n < 1 || !h || !z || !tgt || ((mean == nullptr) != (stdv == nullptr)))
     return KIN_ERR_INVALID_ARG;
   cudaStream_t st = (cudaStream_t)stream;
-  k_targets<<<blocks(n), 256, 0, st>>>(n, nz, h, z, tgt);
-  if (mean) k_standardise<<<blocks(n * (1 + nz)), 256, 0, st>>>(n, 1 + nz, tgt, mean, stdv);
+  k_targets<<<row_blocks(n), FEAT_THREADS, 0, st>>>(n, nz, h, z, mean, stdv, tgt);
   KIN_CUDA_TRY(cudaGetLastError());
   return KIN_OK;
 }
@@ -977,9 +1576,22 @@ extern "C" int kin_mlp_predict(kin_mlp *net, int32_t ns, const double *Y, const 
   cudaStream_t st = (cudaStream_t)stream;
   int rc = mlp_reserve(net, n);
   if (rc) return rc;
+  if (mlp_fused(net)) {  // features straight into the BF16 input
+    if ((rc = launch_features(ns, Y, T, P, n, dt, in_mean, in_std, nullptr, net->xb, net->dinp, st)))
+      return rc;
+    Epilogue ep{};
+    ep.mode = EP_UNPACK;
+    ep.mean = out_mean;
+    ep.stdv = out_std;
+    ep.dt = dt;
+    ep.h0 = h0;
+    ep.z0 = z0;
+    return mlp_forward_fused(net, n, st, false, ep);
+  }
   // features straight into the f32 input block (din <= dinp), then pack in place
-  k_features<<<blocks(n), 256, 0, st>>>(n, ns, Y, T, P, dt, in_mean, in_std, net->dH);
-  if ((rc = mlp_pack(net, net->dH, n, st)) || (rc = mlp_forward_packed(net, n, st))) return rc;
+  if ((rc = launch_features(ns, Y, T, P, n, dt, in_mean, in_std, net->dH, nullptr, 0, st)) ||
+      (rc = mlp_pack(net, net->dH, n, st)) || (rc = mlp_forward_packed(net, n, st)))
+    return rc;
   k_unpack_prediction<<<blocks(n), 256, 0, st>>>(n, net->dout, net->doutp, net->y, out_mean,
                                                  out_std, dt, h0, z0);
   KIN_CUDA_TRY(cudaGetLastError());
