@@ -19,13 +19,27 @@
 // dimension grows until Saad's leading error term of every product taken
 // from it, h beta (h h_{m+1,m}) c_k |e_m^T phi_{k+1}(h H_m) e1| in the
 // step's error weights, is at most kappa, or the space is exhausted.
-// phi_1..phi_p(tau H_m) e1 are columns of the exponential of the augmented
-// matrix [[tau H_m, e1, 0], [0, 0, I], [0, 0, 0]], computed by scaling and
-// squaring with the (6,6) Pade approximant and a partial-pivoting LU.  (The
-// paper uses a (10,10) Caratheodory-Fejer rational approximant of exp on
-// the negative real axis instead; scaling and squaring holds for any
-// spectrum, including the positive eigenvalues of igniting states.)  Step
-// size control: Hairer-Norsett-Wanner on the embedded difference.
+// phi_1..phi_p(tau H_m) e1 come with exp(tau H_m) from scaling and squaring:
+// at A = 2^-s tau H_m with ||A||_1 <= 1/4 by their Taylor series (the powers
+// A^j e1 serve all phi_k at once), then s doublings
+//   F <- 2 F + F F,  phi_k <- 2^-k (phi_k + F phi_k + sum_{j=1..k} phi_j / (k-j)!)
+// with F = E - I, so that the slow modes of a stiff matrix, tiny after the
+// scaling, are not rounded against the identity.  These are the blocks of
+// squaring the exponential of the augmented matrix [[A, e1, 0], [0, 0, I],
+// [0, 0, 0]] without its known rows.  (The paper uses
+// a (10,10) Caratheodory-Fejer rational approximant of exp on the negative
+// real axis instead; scaling and squaring holds for any spectrum, including
+// the positive eigenvalues of igniting states.)  Step size control:
+// Hairer-Norsett-Wanner on the embedded difference.
+//
+// What bounds the kernel is the FP64 unit, and the matrix functions are most
+// of its work: a space of 2.3 vectors on average, so F and the phi_k are a few
+// entries per lane and the cost is the number of FP64 instructions in a
+// doubling.  The squared augmented matrix with its Pade denominator took
+// 1150 of them per evaluation and eleven evaluations a step; the blocks take
+// 300, and the estimate's evaluation at the accepted dimension also gives the
+// step's products (phi_1 at h/2 is the state before the last doubling), so
+// seven evaluations remain.
 #include <cuda_runtime.h>
 
 #include <cmath>
@@ -44,53 +58,51 @@ constexpr int XL = 32;
 using XG = Grp<XL>;
 constexpr int XWR = XG::WR;
 using XV = WVecT<XWR>;
-constexpr int XKP = 5;  // augmented columns: phi_1 .. phi_5
+constexpr int XKP = 5;  // phi_1 .. phi_5 at most
+constexpr int XTERMS = 13;  // Taylor terms: (1/4)^14 / 14! < 2^-64
 
-// Pade (6,6) coefficients of exp: c_j = (12 - j)! 6! / (12! j! (6 - j)!)
-__device__ __constant__ double PADE6[7] = {1.0,        0.5,          5.0 / 44.0,    1.0 / 66.0,
-                                           1.0 / 792.0, 1.0 / 15840.0, 1.0 / 665280.0};
+__device__ __constant__ double INVFACT[20] = {
+    1.0, 1.0, 1.0 / 2.0, 1.0 / 6.0, 1.0 / 24.0, 1.0 / 120.0, 1.0 / 720.0, 1.0 / 5040.0,
+    1.0 / 40320.0, 1.0 / 362880.0, 1.0 / 3628800.0, 1.0 / 39916800.0, 1.0 / 479001600.0,
+    1.0 / 6227020800.0, 1.0 / 87178291200.0, 1.0 / 1307674368000.0, 1.0 / 20922789888000.0,
+    1.0 / 355687428096000.0, 1.0 / 6402373705728000.0, 1.0 / 121645100408832000.0};
+
+// matrix-function scratch for dimension m: A, two power buffers, two buffers
+// of [F | phi_1 .. phi_p]
+__host__ __device__ constexpr size_t xmf_doubles(size_t m) { return 5 * m * m + 2 * XKP * m; }
 
 // per-warp workspace in global memory (after the Jacobian slot)
 struct XWork {
-  double *V;   // basis: vector j at V + j * N, j <= N
-  double *H;   // Hessenberg, (N + 1) x N, H[i * N + j]
-  double *X, *X2, *X4, *U, *W, *R, *Tm;  // S x S, row-major, ld S
-  double *vt;  // S: solve scratch
-  double *vd;  // N: a vector handed to the matrix-vector product
-  int *ip;     // S pivots
-  int S;
+  double *V;     // basis: vector j at V + j * N, j <= N
+  double *H;     // Hessenberg, (N + 1) x N, H[i * N + j]
+  double *mf;    // matrix-function scratch of any dimension up to N
+  double *half;  // phi_1(tau/2 H) e1
+  double *vd;    // N: a vector handed to the matrix-vector product
+  double *fast;  // shared-memory matrix-function scratch
+  int nfast;     // its size in doubles
 };
 
 __host__ __device__ inline int xS(int N) { return (N + XKP + 2) & ~1; }
 __host__ __device__ inline size_t xslot_doubles(int N) {
-  const size_t S = (size_t)xS(N);
   size_t d = (size_t)warp_slot_mats(sizeof(double)) * N * (N + 1);  // J, E2r, E2i
-  d += 2 * (size_t)(N + 1) * N + 7 * S * S + S + (size_t)N + S;     // V, H, 7 matrices, vt, vd, ip
+  d += 2 * (size_t)(N + 1) * N + xmf_doubles(N) + 2 * (size_t)N;    // V, H, mf, half, vd
   return (d + 31) / 32 * 32;
 }
 
 __device__ XWork carve_xwork(double *slot, int N) {
   XWork w;
-  w.S = xS(N);
   double *p = slot + (size_t)warp_slot_mats(sizeof(double)) * N * (N + 1);
   w.V = p;
   p += (size_t)(N + 1) * N;
   w.H = p;
   p += (size_t)(N + 1) * N;
-  const size_t SS = (size_t)w.S * w.S;
-  w.X = p;
-  w.X2 = p + SS;
-  w.X4 = p + 2 * SS;
-  w.U = p + 3 * SS;
-  w.W = p + 4 * SS;
-  w.R = p + 5 * SS;
-  w.Tm = p + 6 * SS;
-  p += 7 * SS;
-  w.vt = p;
-  p += w.S;
-  w.vd = p;
+  w.mf = p;
+  p += xmf_doubles(N);
+  w.half = p;
   p += N;
-  w.ip = reinterpret_cast<int *>(p);
+  w.vd = p;
+  w.fast = nullptr;
+  w.nfast = 0;
   return w;
 }
 
@@ -141,113 +153,99 @@ __device__ void xmatvec(int N, int ld, const double *J, const double *x, XV &y) 
   }
 }
 
-// C = A B for s x s matrices (ld S)
-__device__ void xmatmul(int s, int S, const double *A, const double *B, double *C) {
-  for (int e = XG::lane(); e < s * s; e += XL) {
-    const int i = e / s, j = e % s;
-    double acc = 0.0;
-    for (int k = 0; k < s; ++k) acc += A[i * S + k] * B[k * S + j];
-    C[i * S + j] = acc;
-  }
-  XG::sync();
-}
-
-// exp(w.X) (s x s) by scaling and squaring with the (6,6) Pade approximant;
-// returns the result's matrix (w.R or w.Tm), or nullptr when the
-// denominator is singular or the norm is not finite
-__device__ const double *xexpm(int s, const XWork &w) {
-  const int S = w.S, lane = XG::lane();
+// exp(tau H_m) and phi_1 .. phi_p (tau H_m) e1: entry (i, c) of the returned
+// m x (m + p) array is F[i][c] = (exp - I)[i][c] for c < m, then
+// phi_{c-m+1}[i]; phi_1 at tau/2 in w.half.  nullptr when the norm is not finite.
+__device__ __noinline__ const double *xphi(int N, int m, int p, double tau, const XWork &w) {
+  const int lane = XG::lane(), cols = m + p, mm = m * m, nz = m * cols;
+  double *buf = xmf_doubles(m) <= (size_t)w.nfast ? w.fast : w.mf;
+  double *A = buf, *T0 = buf + mm, *T1 = buf + 2 * mm, *Z = buf + 3 * mm, *Zn = Z + m * (m + XKP);
   double nrm = 0.0;
-  for (int c = lane; c < s; c += XL) {
+  for (int c = lane; c < m; c += XL) {
     double cs = 0.0;
-    for (int i = 0; i < s; ++i) cs += fabs(w.X[i * S + c]);
+    for (int i = 0; i <= c + 1 && i < m; ++i) cs += fabs(tau * w.H[i * N + c]);
     nrm = fmax(nrm, cs);
+    if (!isfinite(cs)) nrm = INFINITY;
   }
 #pragma unroll
   for (int o = XL / 2; o > 0; o >>= 1) nrm = fmax(nrm, __shfl_xor_sync(XG::mask(), nrm, o, XL));
   if (!isfinite(nrm)) return nullptr;
   int sq = 0;
-  while (nrm > 0.25 && sq < 1100) {  // ||X / 2^sq||_1 <= 1/4 (finite norms stop well before)
+  while (nrm > 0.25 && sq < 1100) {  // finite norms stop well before
     nrm *= 0.5;
     ++sq;
   }
   const double sc = ldexp(1.0, -sq);
-  for (int e = lane; e < s * s; e += XL) w.X[(e / s) * S + e % s] *= sc;
-  XG::sync();
-  xmatmul(s, S, w.X, w.X, w.X2);
-  xmatmul(s, S, w.X2, w.X2, w.X4);
-  // W = c1 I + c3 X2 + c5 X4, U = X W
-  for (int e = lane; e < s * s; e += XL) {
-    const int i = e / s, j = e % s, q = i * S + j;
-    w.W[q] = PADE6[3] * w.X2[q] + PADE6[5] * w.X4[q] + (i == j ? PADE6[1] : 0.0);
+  for (int e = lane; e < mm; e += XL) {
+    const int i = e / m, c = e - i * m;
+    // upper Hessenberg: Arnoldi writes no other entry
+    A[e] = i <= c + 1 ? tau * w.H[i * N + c] * sc : 0.0;
+    T0[e] = i == c ? 1.0 : 0.0;
   }
-  XG::sync();
-  xmatmul(s, S, w.X, w.W, w.U);
-  xmatmul(s, S, w.X2, w.X4, w.Tm);  // X6
-  // V = c0 I + c2 X2 + c4 X4 + c6 X6; numerator V + U (R), denominator V - U (W)
-  for (int e = lane; e < s * s; e += XL) {
-    const int i = e / s, j = e % s, q = i * S + j;
-    const double v = PADE6[2] * w.X2[q] + PADE6[4] * w.X4[q] + PADE6[6] * w.Tm[q] +
-                     (i == j ? PADE6[0] : 0.0);
-    w.R[q] = v + w.U[q];
-    w.W[q] = v - w.U[q];
+  for (int e = lane; e < nz; e += XL) {
+    const int i = e / cols, c = e - i * cols;
+    Z[e] = (c >= m && i == 0) ? INVFACT[c - m + 1] : 0.0;
   }
+  if (sq == 0)
+    for (int i = lane; i < m; i += XL) w.half[i] = i == 0 ? 1.0 : 0.0;
   XG::sync();
-  if (warp_lu_real<XL, double>(s, S, w.W, w.ip)) return nullptr;
-  for (int c = 0; c < s; ++c) {  // Tm = W^-1 R, column by column
-    XV x;
-#pragma unroll
-    for (int r = 0; r < XWR; ++r) {
-      const int g = lane + XL * r;
-      x.v[r] = g < s ? w.R[g * S + c] : 0.0;
+  double hpow = 1.0;
+#pragma unroll 1
+  for (int j = 1; j <= XTERMS; ++j) {  // T1 = A T0 = A^j
+    for (int e = lane; e < mm; e += XL) {
+      const int i = e / m, c = e - i * m;
+      double s = 0.0;
+      for (int q = i > 0 ? i - 1 : 0; q < m; ++q) s = fma(A[i * m + q], T0[q * m + c], s);
+      T1[e] = s;
     }
-    warp_solve_real<XL, double>(s, S, w.W, w.ip, w.vt, x);
-#pragma unroll
-    for (int r = 0; r < XWR; ++r) {
-      const int g = lane + XL * r;
-      if (g < s) w.Tm[g * S + c] = x.v[r];
+    XG::sync();
+    for (int e = lane; e < nz; e += XL) {
+      const int i = e / cols, c = e - i * cols;
+      Z[e] = c < m ? fma(T1[i * m + c], INVFACT[j], Z[e])
+                   : fma(T1[i * m], INVFACT[j + c - m + 1], Z[e]);
     }
+    hpow *= 0.5;
+    if (sq == 0)
+      for (int i = lane; i < m; i += XL) w.half[i] = fma(T1[i * m] * hpow, INVFACT[j + 1], w.half[i]);
+    double *t = T0;
+    T0 = T1;
+    T1 = t;
+    XG::sync();
   }
-  XG::sync();
-  double *a = w.Tm, *b = w.R;
-  for (int i = 0; i < sq; ++i) {
-    xmatmul(s, S, a, a, b);
-    double *t = a;
-    a = b;
-    b = t;
+#pragma unroll 1
+  for (int d = 0; d < sq; ++d) {
+    if (d == sq - 1)
+      for (int i = lane; i < m; i += XL) w.half[i] = Z[i * cols + m];
+    for (int e = lane; e < nz; e += XL) {
+      const int i = e / cols, c = e - i * cols;
+      const double *row = Z + i * cols;
+      double s = c < m ? 2.0 * row[c] : row[c];
+      for (int q = 0; q < m; ++q) s = fma(row[q], Z[q * cols + c], s);
+      if (c >= m) {
+        const int k = c - m + 1;
+        for (int q = 1; q <= k; ++q) s = fma(row[m + q - 1], INVFACT[k - q], s);
+        // 2^-k, exact: by the exponent's own multiplication
+        s *= __hiloint2double((1023 - k) << 20, 0);
+      }
+      Zn[e] = s;
+    }
+    double *t = Z;
+    Z = Zn;
+    Zn = t;
+    XG::sync();
   }
-  return a;
+  return Z;
 }
 
-// phi_1 .. phi_p (tau H_m) e1: the exponential of the augmented matrix;
-// phi_k is column m + k - 1 (rows 0 .. m-1) of the returned matrix
-__device__ const double *xphi(int N, int m, int p, double tau, const XWork &w) {
-  const int s = m + p, S = w.S;
-  for (int e = XG::lane(); e < s * s; e += XL) {
-    const int i = e / s, j = e % s;
-    double v = 0.0;
-    if (i < m && j < m && i <= j + 1)  // upper Hessenberg: Arnoldi writes no other entry
-      v = tau * w.H[i * N + j];
-    else if (i == 0 && j == m)
-      v = 1.0;
-    else if (i >= m && j == i + 1)
-      v = 1.0;
-    w.X[i * S + j] = v;
-  }
-  XG::sync();
-  return xexpm(s, w);
-}
-
-// D beta V_m phi_k e1 with phi_k read from the exponential E (column m+k-1)
-__device__ void xproduct(int N, int m, double beta, const XWork &w, const double *E, int k,
+// D beta V_m phi with phi's component i at ph[i * stride]
+__device__ void xproduct(int N, int m, double beta, const XWork &w, const double *ph, int stride,
                          const XV &scal, XV &out) {
-  const int S = w.S;
 #pragma unroll
   for (int r = 0; r < XWR; ++r) {
     const int g = XG::lane() + XL * r;
     double s = 0.0;
     if (g < N)
-      for (int i = 0; i < m; ++i) s += w.V[i * N + g] * E[i * S + m + k - 1];
+      for (int i = 0; i < m; ++i) s += w.V[i * N + g] * ph[i * stride];
     out.v[r] = scal.v[r] * (beta * s);
   }
 }
@@ -260,10 +258,11 @@ struct XProducts {
 
 // Arnoldi in the error-weighted inner product (on D^-1 J D from D^-1 v,
 // D = diag(scal)) with the stopping rule; returns m (0 for v = 0), -1 when
-// a matrix function failed; beta out
+// a matrix function failed; beta and the matrix functions at the returned
+// dimension (xphi's array, kmax + 1 phi functions) out
 __device__ int xarnoldi(int N, int ld, const double *J, const XV &v, double h,
                         const XProducts &pr, const XV &scal, double kappa, const XWork &w,
-                        double &beta) {
+                        double &beta, const double *&Z) {
   const int lane = XG::lane();
   XV q;
 #pragma unroll
@@ -299,18 +298,20 @@ __device__ int xarnoldi(int N, int ld, const double *J, const XV &v, double h,
     const int m = j + 1;
     if (hn <= 1e-13 * nw || m == N) {
       XG::sync();
-      return m;
+      Z = xphi(N, m, pr.kmax + 1, h, w);
+      return Z ? m : -1;
     }
 #pragma unroll
     for (int r = 0; r < XWR; ++r) x.v[r] = x.v[r] / hn;
     xstore(N, w.V + (size_t)(j + 1) * N, x);
     XG::sync();
-    const double *E = xphi(N, m, pr.kmax + 1, h, w);
+    Z = xphi(N, m, pr.kmax + 1, h, w);
     // a failed matrix function or a non-finite entry gives no estimate: keep growing
-    double lead = E ? 0.0 : NAN;
-    if (E)
+    double lead = Z ? 0.0 : NAN;
+    if (Z)
       for (int t = 0; t < pr.np; ++t) {
-        const double v = pr.c[t] * fabs(E[(m - 1) * w.S + m + pr.k[t]]);  // phi_{k+1}
+        const double v =
+            pr.c[t] * fabs(Z[(m - 1) * (m + pr.kmax + 1) + m + pr.k[t]]);  // phi_{k+1}
         lead = isnan(v) || isnan(lead) ? NAN : fmax(lead, v);
       }
     // v_{m+1} has unit 2-norm in the scaled space: weighted RMS 1/sqrt(N)
@@ -318,7 +319,7 @@ __device__ int xarnoldi(int N, int ld, const double *J, const XV &v, double h,
     XG::sync();
     if (est <= kappa) return m;
   }
-  return N;
+  return -1;  // not reached: the space is exhausted at m = N
 }
 
 struct XParams {
@@ -356,21 +357,17 @@ __device__ int xstep(const MechView &m, const WarpBuf<double> &b, double P, cons
   nf = 0;
   kdim = 0;
   double beta;
+  const double *Z = nullptr;
   XV half, full, U, F, D, q1, q3, q4, r3, r4;
-  int mk = xarnoldi(N, ld, J, fy, h, PF, scal, kappa, w, beta);
+  int mk = xarnoldi(N, ld, J, fy, h, PF, scal, kappa, w, beta, Z);
   if (mk < 0) return 2;
   kdim += mk;
   if (mk == 0) {
 #pragma unroll
     for (int r = 0; r < XWR; ++r) half.v[r] = full.v[r] = 0.0;
   } else {
-    const double *E = xphi(N, mk, 1, 0.5 * h, w);
-    if (!E) return 2;
-    xproduct(N, mk, beta, w, E, 1, scal, half);
-    XG::sync();
-    E = xphi(N, mk, 1, h, w);
-    if (!E) return 2;
-    xproduct(N, mk, beta, w, E, 1, scal, full);
+    xproduct(N, mk, beta, w, w.half, 1, scal, half);
+    xproduct(N, mk, beta, w, Z + mk, mk + PF.kmax + 1, scal, full);
     XG::sync();
   }
 #pragma unroll
@@ -378,18 +375,17 @@ __device__ int xstep(const MechView &m, const WarpBuf<double> &b, double P, cons
   nf++;
   if (warp_chem<XL, double>(m, b, P, U, F, false)) return 1;
   xremainder(N, ld, J, U, y, F, fy, w, D);
-  mk = xarnoldi(N, ld, J, D, h, PD2, scal, kappa, w, beta);
+  mk = xarnoldi(N, ld, J, D, h, PD2, scal, kappa, w, beta, Z);
   if (mk < 0) return 2;
   kdim += mk;
   if (mk == 0) {
 #pragma unroll
     for (int r = 0; r < XWR; ++r) q1.v[r] = q3.v[r] = q4.v[r] = 0.0;
   } else {
-    const double *E = xphi(N, mk, 4, h, w);
-    if (!E) return 2;
-    xproduct(N, mk, beta, w, E, 1, scal, q1);
-    xproduct(N, mk, beta, w, E, 3, scal, q3);
-    xproduct(N, mk, beta, w, E, 4, scal, q4);
+    const int ld2 = mk + PD2.kmax + 1;
+    xproduct(N, mk, beta, w, Z + mk, ld2, scal, q1);
+    xproduct(N, mk, beta, w, Z + mk + 2, ld2, scal, q3);
+    xproduct(N, mk, beta, w, Z + mk + 3, ld2, scal, q4);
     XG::sync();
   }
 #pragma unroll
@@ -397,17 +393,16 @@ __device__ int xstep(const MechView &m, const WarpBuf<double> &b, double P, cons
   nf++;
   if (warp_chem<XL, double>(m, b, P, U, F, false)) return 1;
   xremainder(N, ld, J, U, y, F, fy, w, D);
-  mk = xarnoldi(N, ld, J, D, h, PD3, scal, kappa, w, beta);
+  mk = xarnoldi(N, ld, J, D, h, PD3, scal, kappa, w, beta, Z);
   if (mk < 0) return 2;
   kdim += mk;
   if (mk == 0) {
 #pragma unroll
     for (int r = 0; r < XWR; ++r) r3.v[r] = r4.v[r] = 0.0;
   } else {
-    const double *E = xphi(N, mk, 4, h, w);
-    if (!E) return 2;
-    xproduct(N, mk, beta, w, E, 3, scal, r3);
-    xproduct(N, mk, beta, w, E, 4, scal, r4);
+    const int ld3 = mk + PD3.kmax + 1;
+    xproduct(N, mk, beta, w, Z + mk + 2, ld3, scal, r3);
+    xproduct(N, mk, beta, w, Z + mk + 3, ld3, scal, r4);
     XG::sync();
   }
 #pragma unroll
@@ -548,7 +543,10 @@ __global__ void __launch_bounds__(256) k_integrate_exprb(XArgs a) {
   const int64_t slot = (int64_t)blockIdx.x * (blockDim.x / XL) + grp;  // < slots (launch)
   double *gs = a.scratch + slot * (int64_t)xslot_doubles(N);
   const WarpBuf<double> b = carve_warp_buf<double>(base, N, m.nr, gs);
-  const XWork w = carve_xwork(gs, N);
+  XWork w = carve_xwork(gs, N);
+  // E1's shared memory is free outside the Jacobian's assembly
+  w.fast = b.E1;
+  w.nfast = (int)(warp_e1_bytes(N, sizeof(double)) / sizeof(double));
   unsigned long long *queue = a.totals + 9;
   for (;;) {
     unsigned long long t = 0;
@@ -601,9 +599,9 @@ __global__ void k_exprb_phi(const double *H, int m, int p, double tau, double *o
   XWork w = carve_xwork(scratch, N);
   for (int e = threadIdx.x; e < m * m; e += XL) w.H[(e / m) * N + e % m] = H[e];
   XG::sync();
-  const double *E = xphi(N, m, p, tau, w);
+  const double *Z = xphi(N, m, p, tau, w);
   for (int e = threadIdx.x; e < m * p; e += XL)
-    out[e] = E ? E[(e / p) * w.S + m + e % p] : NAN;  // out[i * p + k - 1] = phi_k[i]
+    out[e] = Z ? Z[(e / p) * (m + p) + m + e % p] : NAN;  // out[i * p + k - 1] = phi_k[i]
 }
 
 // unit entry: the right-hand side (with and without the Jacobian's assembly)

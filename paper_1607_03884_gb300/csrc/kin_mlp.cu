@@ -366,6 +366,9 @@ __global__ void __launch_bounds__(TC_THREADS) k_gemm_tc(int M, int N, int K,
 // their K order are k_gemm_tc's: the same bits.
 // ---------------------------------------------------------------------------
 constexpr int KK_STAGES = 3;
+// eight warps: warps w and w + 4 share TMEM lanes 32 w .. 32 w + 31 and halve
+// the epilogue's columns
+constexpr int KK_THREADS = 256;
 constexpr int KK_STAGE_BYTES = 2 * TC_BM * TC_BK * 2;
 constexpr size_t KK_SMEM = (size_t)KK_STAGES * KK_STAGE_BYTES + 1024;  // two CTAs per SM
 
@@ -472,7 +475,7 @@ __device__ __forceinline__ void tma_box(uint32_t dst, const CUtensorMap *tm, int
       : "memory");
 }
 
-__global__ void __launch_bounds__(TC_THREADS) k_gemm_kk(int64_t M, int N, int K, int *err,
+__global__ void __launch_bounds__(KK_THREADS) k_gemm_kk(int64_t M, int N, int K, int *err,
                                                        const __grid_constant__ CUtensorMap tmA,
                                                        const __grid_constant__ CUtensorMap tmB,
                                                        const __grid_constant__ Epilogue ep) {
@@ -567,11 +570,11 @@ __global__ void __launch_bounds__(TC_THREADS) k_gemm_kk(int64_t M, int N, int K,
   const bool good = __syncthreads_and(done) && !failed;
   float loss = 0.0f;
   if (good) {
-    const int64_t row = m0 + warp * 32 + lane;
+    const int64_t row = m0 + (warp & 3) * 32 + lane;
     const int nc = N - n0 < TC_BN ? N - n0 : TC_BN;
-    for (int c0 = 0; c0 < nc; c0 += 16) {
+    for (int c0 = (warp >> 2) * 16; c0 < nc; c0 += 32) {
       uint32_t v[16];
-      const uint32_t taddr = tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c0;
+      const uint32_t taddr = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)c0;
       asm volatile(
           "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,"
           "%14,%15}, [%16];\n"
@@ -681,22 +684,39 @@ __global__ void k_silu_back(int64_t n, const float *dH, const float *a, float *g
   if (gb) gb[i] = __float2bfloat16(v);
 }
 
-// column sums: out[c] = sum_r g[r][c]; a block per 32 columns, 32 row lanes
-// (a thread per column alone walked 4096 rows in sequence: 300 us)
-__global__ void __launch_bounds__(1024) k_colsum(int64_t M, int N, const float *g, float *out) {
-  __shared__ float part[32][33];
-  const int c = blockIdx.x * 32 + (threadIdx.x & 31), y = threadIdx.x >> 5;
+// column sums: out[c] = sum_r g[r][c]; a cluster of eight CTAs per 32 columns,
+// its partial sums added through distributed shared memory in a fixed order
+// (a thread per column alone walked 4096 rows in sequence)
+constexpr int CS_CTAS = 8, CS_THREADS = 512;
+
+__global__ void __cluster_dims__(CS_CTAS, 1, 1) __launch_bounds__(CS_THREADS)
+    k_colsum(int64_t M, int N, const float *g, float *out) {
+  namespace cg = cooperative_groups;
+  cg::cluster_group cl = cg::this_cluster();
+  __shared__ float part[CS_THREADS / 32][32], mine[32];
+  const int lane = threadIdx.x & 31, y = threadIdx.x >> 5;
+  const int c = (int)(blockIdx.x / CS_CTAS) * 32 + lane;
+  const int64_t step = (int64_t)CS_CTAS * (CS_THREADS / 32);
   float s = 0.0f;
   if (c < N) {
 #pragma unroll 4
-    for (int64_t r = y; r < M; r += 32) s += g[r * N + c];
+    for (int64_t r = (int64_t)cl.block_rank() * (CS_THREADS / 32) + y; r < M; r += step)
+      s += g[r * N + c];
   }
-  part[y][threadIdx.x & 31] = s;
+  part[y][lane] = s;
   __syncthreads();
-  float t = part[threadIdx.x & 31][y];
-  for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-  const int co = blockIdx.x * 32 + y;
-  if ((threadIdx.x & 31) == 0 && co < N) out[co] = t;
+  if (y == 0) {
+    float t = 0.0f;
+    for (int w = 0; w < CS_THREADS / 32; ++w) t += part[w][lane];
+    mine[lane] = t;
+  }
+  cl.sync();
+  if (cl.block_rank() == 0 && y == 0 && c < N) {
+    float t = 0.0f;
+    for (int k = 0; k < CS_CTAS; ++k) t += cl.map_shared_rank(&mine[0], k)[lane];
+    out[c] = t;
+  }
+  cl.sync();
 }
 
 // weight blocks of the network: offset, K, N per layer
@@ -1128,7 +1148,7 @@ static int gemm_kk(const kin_mlp *n, cudaStream_t st, int64_t M, int N, int K,
   CUtensorMap tmA, tmB;
   if (!make_tmap(&tmA, A, M, K, K, true) || !make_tmap(&tmB, B, N, K, K, true)) return KIN_ERR_CUDA;
   const dim3 grid((unsigned)((M + TC_BM - 1) / TC_BM), (unsigned)((N + TC_BN - 1) / TC_BN), 1);
-  k_gemm_kk<<<grid, TC_THREADS, KK_SMEM, st>>>(M, N, K, n->err, tmA, tmB, ep);
+  k_gemm_kk<<<grid, KK_THREADS, KK_SMEM, st>>>(M, N, K, n->err, tmA, tmB, ep);
   KIN_CUDA_TRY(cudaGetLastError());
   return KIN_OK;
 }
@@ -1175,7 +1195,7 @@ static int mlp_grad_fused(kin_mlp *n, int64_t M, const float *T, const int32_t *
     const int K = n->K[l], N = n->N[l];
     gemm(n, st, K, N, (int)M, true, l ? n->hb[l - 1] : n->xb, 1, K, gb, N, 1,
          n->grad + n->woff[l], N, 0);
-    k_colsum<<<blocks(N, 32), 1024, 0, st>>>(M, N, g, n->grad + n->boff[l]);
+    k_colsum<<<CS_CTAS * blocks(N, 32), CS_THREADS, 0, st>>>(M, N, g, n->grad + n->boff[l]);
     if (l == 0) break;
     Epilogue e{};
     e.mode = EP_BACK;
@@ -1220,7 +1240,7 @@ static int mlp_backward(kin_mlp *n, int64_t M, cudaStream_t st) {
     const void *gv = bf ? (const void *)n->gb : (const void *)n->g;
     // dW[i][o] = sum_b h[b][i] g[b][o]
     gemm(n, st, K, N, (int)M, bf, hin, 1, K, gv, N, 1, n->grad + n->woff[l], N, 0);
-    k_colsum<<<blocks(N, 32), 1024, 0, st>>>(M, N, n->g, n->grad + n->boff[l]);
+    k_colsum<<<CS_CTAS * blocks(N, 32), CS_THREADS, 0, st>>>(M, N, n->g, n->grad + n->boff[l]);
     if (l == 0) break;
     // dH[b][i] = sum_o g[b][o] W[i][o]
     const void *W = bf ? (const void *)(n->wb + n->woff[l]) : (const void *)(n->p + n->woff[l]);
