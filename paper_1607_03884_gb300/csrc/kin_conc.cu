@@ -150,68 +150,71 @@ void conc_counts(const ConcStructure &S, int64_t *out) {
   out[3] = sol;
 }
 
-// offsets into the device int table: var | posn | lp | li | up | uj | cp | ci
 struct ConcArgs {
   KernelArgs a;
-  int N, k0, posT, posV;
-  const int *ctab;
+  int N, posT, posV;
+  const int *ctab;  // var [N], posn [ns - 1]
   const double *aw;
-  int o_posn, o_lp, o_li, o_up, o_uj, o_cp, o_ci;
 };
 
-template <int L, typename LT>
-__global__ void __launch_bounds__(256) k_integrate_conc(ConcArgs ca) {
-  using G = Grp<L>;
-  constexpr int WR = G::WR;
-  extern __shared__ double smem[];
+template <typename LT>
+__global__ void __launch_bounds__(TEAM_MAX *TEAM_NT, 1) k_integrate_conc(ConcArgs ca) {
+  using G = Grp<32>;
+  extern __shared__ __align__(16) unsigned char team_smem[];
   const KernelArgs &a = ca.a;
   const MechView m = make_view(a.L, a.tab, a.itab);
-  ConcView cv;
-  cv.N = ca.N;
-  cv.k0 = ca.k0;
-  cv.posT = ca.posT;
-  cv.posV = ca.posV;
-  cv.var = ca.ctab;
-  cv.posn = ca.ctab + ca.o_posn;
-  cv.lp = ca.ctab + ca.o_lp;
-  cv.li = ca.ctab + ca.o_li;
-  cv.up = ca.ctab + ca.o_up;
-  cv.uj = ca.ctab + ca.o_uj;
-  cv.cp = ca.ctab + ca.o_cp;
-  cv.ci = ca.ctab + ca.o_ci;
-  cv.aw = ca.aw;
-  const int N = cv.N, ns = m.ns, in = ns - 1, lane = G::lane(), grp = (int)(threadIdx.x / L);
+  const ConcView cv{ca.N, ca.posT, ca.posV, ca.ctab, ca.ctab + ca.N, ca.aw};
+  const int N = cv.N, ns = m.ns, in = ns - 1, lane = G::lane(), warp = (int)(threadIdx.x / 32);
+  const int team = warp / TEAM_WARPS, wt = warp % TEAM_WARPS;
   const int64_t n = a.rp.n;
-  char *base = reinterpret_cast<char *>(smem) + (size_t)grp * warp_buf_bytes(N, m.nr, sizeof(LT));
-  const int64_t slot = (int64_t)blockIdx.x * (blockDim.x / L) + grp;  // < gslots (launch)
-  LT *Jg = reinterpret_cast<LT *>(a.gscratch) +
-           slot * (int64_t)warp_slot_mats(sizeof(LT)) * N * (N + 1);
-  const WarpBuf<LT> b = carve_warp_buf<LT>(base, N, m.nr, Jg);
-  const ConcSys<L, LT> sys{&m, &cv};
+  // the tables' Jacobian columns are elements of phi (kin_conc_create)
+  const HotTables h = stage_hot(a.L, a.hot, a.hot_smem != 0, team_smem);
+  const size_t hb = a.hot_smem ? hot_offsets(a.L).bytes : 0;
+  const size_t tb = team_bytes(a.L, N, sizeof(LT));
+  const int64_t slot = (int64_t)blockIdx.x * (blockDim.x / TEAM_NT) + team;  // < gslots (launch)
+  const TeamBuf<LT> t = carve_team<LT>(
+      a.L, team_smem + hb + team * tb, team, N,
+      reinterpret_cast<unsigned char *>(a.gscratch) +
+          slot * (int64_t)warp_slot_mats(sizeof(LT)) * N * (N + 1) * (int64_t)sizeof(LT));
+  const TeamConc<LT> f{m, h, t, cv};
+  if (wt != 0) {  // workers: a part of each command until the leader is done
+    for (;;) {
+      named_sync(t.bar, TEAM_NT);
+      const int cmd = t.ctl->cmd;
+      if (cmd == TEAM_QUIT) return;
+      team_exec<LT>(cmd, wt, f);
+      named_sync(t.bar, TEAM_NT);
+    }
+  }
+  const TeamSys<LT, TeamConc<LT>> sys{f};
+  WarpBuf<LT> b{};
+  b.J = t.J;
   unsigned long long *queue = a.totals + 9;
-  WStateT<WR> w;
+  WStateT<2> w;
   StepState s;
   for (;;) {
-    unsigned long long t = 0;
-    if (lane == 0) t = atomicAdd(queue, 1ull);
-    t = G::bcast(t, 0);
-    if (t >= (unsigned long long)n) break;
+    unsigned long long q = 0;
+    if (lane == 0) q = atomicAdd(queue, 1ull);
+    q = G::bcast(q, 0);
+    if (q >= (unsigned long long)n) break;
     int64_t idx = 0;
-    if (lane == 0) idx = state_of(a, (int64_t)t);
+    if (lane == 0) idx = state_of(a, (int64_t)q);
     idx = G::bcast(idx, 0);
     if (idx < 0) continue;
     const double P = a.P[idx], T0 = a.T[idx];
+    if (lane == 0) t.ctl->P = P;
+    __syncwarp();
     // phi per unit mass: n_k = Y_k / W_k, V = Ru T sum_k (Y_k / W_k) / P
     double sS = 0.0;
 #pragma unroll
-    for (int r = 0; r < WR; ++r) {
-      const int k = lane + L * r;
+    for (int r = 0; r < 2; ++r) {
+      const int k = lane + 32 * r;
       if (k < ns) sS += a.Y[(int64_t)k * n + idx] * m.invW[k];
     }
     sS = G::sum(sS);
 #pragma unroll
-    for (int r = 0; r < WR; ++r) {
-      const int g = lane + L * r;
+    for (int r = 0; r < 2; ++r) {
+      const int g = lane + 32 * r;
       const int v = g < N ? cv.var[g] : -1;
       w.y.v[r] = (v == 0)   ? T0
                  : (v == 1) ? RU * T0 * sS / P
@@ -219,15 +222,15 @@ __global__ void __launch_bounds__(256) k_integrate_conc(ConcArgs ca) {
                             : 0.0;
     }
     // every attempt ends the loop or counts a step; max_steps bounds it
-    bool done = warp_init_sys<L, LT, false>(sys, b, P, w, s, a.rp, idx);
-    while (!done) done = warp_step_sys<L, LT, false>(sys, b, P, w, s, a.rp, idx);
+    bool done = warp_init_sys<32, LT, false>(sys, b, P, w, s, a.rp, idx);
+    while (!done) done = warp_step_sys<32, LT, false>(sys, b, P, w, s, a.rp, idx);
     // back to mass fractions: the bath gas's moles close P V = n Ru T; Y_k is
     // W_k n_k over the mixture's mass
-    const double T1 = elem<L>(w.y, cv.posT), V1 = elem<L>(w.y, cv.posV);
+    const double T1 = elem<32>(w.y, cv.posT), V1 = elem<32>(w.y, cv.posV);
     double sn = 0.0, sm = 0.0;
 #pragma unroll
-    for (int r = 0; r < WR; ++r) {
-      const int g = lane + L * r;
+    for (int r = 0; r < 2; ++r) {
+      const int g = lane + 32 * r;
       const int v = g < N ? cv.var[g] : -1;
       if (v >= 2) {
         sn += w.y.v[r];
@@ -239,63 +242,29 @@ __global__ void __launch_bounds__(256) k_integrate_conc(ConcArgs ca) {
     const double nin = P * V1 / (RU * T1) - sn;
     const double imass = 1.0 / (sm + m.W[in] * nin);
 #pragma unroll
-    for (int r = 0; r < WR; ++r) {
-      const int g = lane + L * r;
+    for (int r = 0; r < 2; ++r) {
+      const int g = lane + 32 * r;
       const int v = g < N ? cv.var[g] : -1;
       if (v >= 2) a.Y[(int64_t)(v - 2) * n + idx] = m.W[v - 2] * w.y.v[r] * imass;
     }
     if (lane == 0) {
       a.T[idx] = T1;
       a.Y[(int64_t)in * n + idx] = m.W[in] * nin * imass;
-      if (a.status) a.status[idx] = s.status;
-      if (a.counters) {
-        const int32_t c[8] = {s.nstep, s.naccpt, s.nrejct, s.nfcn, s.njac, s.ndec, s.nsol,
-                              s.status};
-        for (int q = 0; q < 8; ++q) a.counters[(int64_t)q * n + idx] = c[q];
-      }
-      const unsigned long long c7[7] = {
-          (unsigned long long)s.nstep, (unsigned long long)s.naccpt, (unsigned long long)s.nrejct,
-          (unsigned long long)s.nfcn,  (unsigned long long)s.njac,   (unsigned long long)s.ndec,
-          (unsigned long long)s.nsol};
-      for (int q = 0; q < 7; ++q) atomicAdd(a.totals + q, c7[q]);
-      if (s.status) atomicAdd(a.totals + 7, 1ull);
-      atomicMax(a.totals + 8, (unsigned long long)s.nstep);
     }
-    G::sync();
+    store_counts<32>(s, a, idx);
   }
+  sys.post(TEAM_QUIT);
 }
 
-template <int L, typename LT>
-int launch_conc(const ConcArgs &ca, cudaStream_t st, int sms) {
-  using G = Grp<L>;
-  const KernelArgs &a = ca.a;
-  if (ca.N > G::CAP) return KIN_ERR_UNSUPPORTED;
+template <typename LT>
+int launch_conc(ConcArgs ca, cudaStream_t st, int sms) {
+  KernelArgs &a = ca.a;
   if (!a.gscratch || a.gslots < 1) return KIN_ERR_UNSUPPORTED;
-  const size_t budget = 227 * 1024, per_grp = warp_buf_bytes(ca.N, a.L.nr, sizeof(LT));
-  auto kern = k_integrate_conc<L, LT>;
-  // the block size (1 to 8 warps) that keeps the most warps resident per SM
-  int warps = 0, per_sm = 0;
-  for (int wp = 8; wp >= 1; wp >>= 1) {
-    const size_t smw = (size_t)wp * (32 / L) * per_grp;
-    if (smw > budget) continue;
-    KIN_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smw));
-    int nb = 0;
-    KIN_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, 32 * wp, smw));
-    if (nb * wp > per_sm * warps) {
-      warps = wp;
-      per_sm = nb;
-    }
-  }
-  if (warps < 1 || per_sm < 1) return KIN_ERR_UNSUPPORTED;
-  const size_t sm = (size_t)warps * (32 / L) * per_grp;
-  KIN_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-  int64_t grid = (int64_t)sms * per_sm;
-  const int64_t per_block = (int64_t)warps * (32 / L);
-  const int64_t need = (a.rp.n + per_block - 1) / per_block;
-  if (grid > need) grid = need;
-  if (grid * per_block > a.gslots) grid = a.gslots / per_block;  // one J slot per group
-  if (grid < 1) return KIN_ERR_UNSUPPORTED;
-  kern<<<(unsigned)grid, 32 * warps, sm, st>>>(ca);
+  TeamLaunch g;
+  if (!team_shape(a, ca.N, sizeof(LT), sms, g)) return KIN_ERR_UNSUPPORTED;
+  auto kern = k_integrate_conc<LT>;
+  KIN_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g.smem));
+  kern<<<g.grid, g.threads, g.smem, st>>>(ca);
   KIN_CUDA_TRY(cudaGetLastError());
   return KIN_OK;
 }
@@ -310,9 +279,9 @@ struct kin_conc {
   int *d_itab = nullptr;
   int *d_ctab = nullptr;
   double *d_aw = nullptr;  // [N] factor on atol per element
-  int o_posn = 0, o_lp = 0, o_li = 0, o_up = 0, o_uj = 0, o_cp = 0, o_ci = 0;
   unsigned long long *d_totals = nullptr;
   void *d_gscratch = nullptr;
+  unsigned char *d_hot = nullptr;  // the teams' tables
   int64_t gslots = 0;
   cudaStream_t last_stream = nullptr;
 };
@@ -338,6 +307,7 @@ extern "C" void kin_conc_destroy(kin_conc *c) {
   cudaFree(c->d_aw);
   cudaFree(c->d_totals);
   cudaFree(c->d_gscratch);
+  cudaFree(c->d_hot);
   delete c;
 }
 
@@ -373,28 +343,20 @@ extern "C" int kin_conc_create(const kin_mech_desc *desc, kin_conc **out) {
   rk.ic2m1 = 1.0 / (rk.c2 - 1.0);
   rk.ic1mc2 = 1.0 / (rk.c1 - rk.c2);
   KIN_CUDA_TRY(cudaMemcpyToSymbol(RC, &rk, sizeof rk));
-  // device int table: var | posn | lp | li | up | uj | cp | ci
+  // device int table: var | posn
   const int N = S.N, ns = desc->ns;
   std::vector<int> ct(S.var.begin(), S.var.end());
   kin_conc *c = new kin_conc();
-  c->o_posn = (int)ct.size();
-  ct.resize(ct.size() + (ns - 1));
+  ct.resize(N + (ns - 1));
   for (int g = 0; g < N; ++g)
-    if (S.var[g] >= 2) ct[c->o_posn + S.var[g] - 2] = g;
-  auto append = [&](const std::vector<int> &v) {
-    const int o = (int)ct.size();
-    ct.insert(ct.end(), v.begin(), v.end());
-    if (v.empty()) ct.push_back(0);
-    return o;
-  };
-  c->o_lp = append(S.lp);
-  c->o_li = append(S.li);
-  c->o_up = append(S.up);
-  c->o_uj = append(S.uj);
-  c->o_cp = append(S.cp);
-  c->o_ci = append(S.ci);
+    if (S.var[g] >= 2) ct[N + S.var[g] - 2] = g;
   c->L = L;
   c->S = S;
+  // the teams' tables, the Jacobian rows' columns as elements of phi (the bath
+  // gas, the last species, has none)
+  std::vector<unsigned char> hot = build_hot(L, dt, it);
+  for (size_t x = hot_offsets(L).col; x < hot_offsets(L).col + L.nslots + L.neff; ++x)
+    if (hot[x] < ns - 1) hot[x] = (unsigned char)ct[N + hot[x]];
   // the moles' absolute tolerance is atol / W_k (T and V: atol)
   std::vector<double> aw(N, 1.0);
   for (int g = 0; g < N; ++g)
@@ -417,6 +379,7 @@ extern "C" int kin_conc_create(const kin_mech_desc *desc, kin_conc **out) {
       cudaMalloc(&c->d_ctab, sizeof(int) * ct.size()) != cudaSuccess ||
       cudaMalloc(&c->d_aw, sizeof(double) * N) != cudaSuccess ||
       cudaMalloc(&c->d_totals, sizeof(unsigned long long) * 16) != cudaSuccess ||
+      cudaMalloc(&c->d_hot, hot.size()) != cudaSuccess ||
       cudaMalloc(&c->d_gscratch, gbytes) != cudaSuccess) {
     (void)cudaGetLastError();
     kin_conc_destroy(c);
@@ -428,6 +391,7 @@ extern "C" int kin_conc_create(const kin_mech_desc *desc, kin_conc **out) {
           cudaSuccess ||
       cudaMemcpy(c->d_ctab, ct.data(), sizeof(int) * ct.size(), cudaMemcpyHostToDevice) !=
           cudaSuccess ||
+      cudaMemcpy(c->d_hot, hot.data(), hot.size(), cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaMemcpy(c->d_aw, aw.data(), sizeof(double) * N, cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaMemset(c->d_totals, 0, sizeof(unsigned long long) * 16) != cudaSuccess) {
     (void)cudaGetLastError();
@@ -499,8 +463,9 @@ extern "C" int kin_integrate_conc(kin_conc *c, double *Y, double *T, const doubl
   a.order = o.order;
   a.gscratch = c->d_gscratch;
   a.gslots = c->gslots;
+  a.hot = c->d_hot;
+  a.hot_smem = 0;
   ca.N = c->S.N;
-  ca.k0 = c->S.k0;
   ca.posT = ca.posV = -1;
   for (int g = 0; g < ca.N; ++g) {
     if (c->S.var[g] == 0) ca.posT = g;
@@ -508,14 +473,7 @@ extern "C" int kin_integrate_conc(kin_conc *c, double *Y, double *T, const doubl
   }
   ca.ctab = c->d_ctab;
   ca.aw = c->d_aw;
-  ca.o_posn = c->o_posn;
-  ca.o_lp = c->o_lp;
-  ca.o_li = c->o_li;
-  ca.o_up = c->o_up;
-  ca.o_uj = c->o_uj;
-  ca.o_cp = c->o_cp;
-  ca.o_ci = c->o_ci;
-  return o.lu_fp32 ? launch_conc<32, float>(ca, st, sms) : launch_conc<32, double>(ca, st, sms);
+  return o.lu_fp32 ? launch_conc<float>(ca, st, sms) : launch_conc<double>(ca, st, sms);
 }
 
 extern "C" int kin_conc_get_stats(kin_conc *c, int64_t *out) {

@@ -11,6 +11,9 @@ namespace kin {
 // Validate a mechanism description and build its device tables on the host.
 int build_tables(const kin_mech_desc *d, MechLayout &L, std::vector<double> &dt,
                  std::vector<int> &it);
+// The team kernels' tables (kin_team.cuh, HotOffsets) from the device tables.
+std::vector<unsigned char> build_hot(const MechLayout &L, const std::vector<double> &dt,
+                                     const std::vector<int> &it);
 // Upload the Radau constants to every kernel translation unit, once per device.
 int ensure_constants(int dev);
 // Launch the integration kernel that matches the options and species count.

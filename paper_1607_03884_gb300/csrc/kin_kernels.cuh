@@ -45,6 +45,8 @@ struct KernelArgs {
   const int32_t *order;  // slot -> state permutation or null (identity)
   void *gscratch;        // WARP: per-group Jacobian slots (N x (N+1) doubles each)
   int64_t gslots;        // number of slots in gscratch
+  const unsigned char *hot;  // WARP with 32 lanes: the teams' tables (kin_team.cuh)
+  int hot_smem;              // copied to shared memory by each block
 };
 
 // The state a slot carries: order[slot] when an order is given, else the
@@ -149,8 +151,17 @@ __device__ __forceinline__ void bind_scratch(Work<MAXN, LT> &w, const KernelArgs
 #endif
 }
 
-template <int MAXN, typename LT, bool FDJ>
-__global__ void KIN_THREAD_BOUNDS k_integrate_plain(KernelArgs a) {
+// Resident 64-thread blocks per SM that a PLAIN kernel's registers allow.  A
+// batch that fills the chip takes KIN_THREAD_MIN_BLOCKS (48 registers: hiding
+// latency is worth more than spills); one that leaves SMs with fewer blocks
+// than that anyway takes the registers they leave free (168, 96 or 72), which
+// spill less.  Ordered mixed H2 states, dt = 1e-4 s, ms, with 48 registers and
+// with the free ones: FP64 50021: 315, 304, 80000: 793, 515, 131072: 1153, 896;
+// FP32 50021: 240, 222, 80000: 525, 364, 131072: 772, 617.
+constexpr int PLAIN_BLOCKS_FEW = 6, PLAIN_BLOCKS_MID = 10, PLAIN_BLOCKS_MANY = 14;
+
+template <int MAXN, typename LT, bool FDJ, int MINB>
+__global__ void __launch_bounds__(64, MINB) k_integrate_plain(KernelArgs a) {
   extern __shared__ double smem[];
   const MechView m = KIN_THREAD_VIEW(a, smem);
   const int64_t slot = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -262,26 +273,40 @@ __global__ void __launch_bounds__(COOP_NT, 8) k_integrate_coop(KernelArgs a) {
 
 // PLAIN batches of at most this many states go to k_integrate_coop: its time
 // grows with the batch, the per-thread kernel's is flat (a chain of FP64
-// latencies) until its warps fill the chip.  H2, dt = 1e-6 / 1e-4 s, ms,
-// coop against per thread: FP64 2048: 40 / 60 against 156 / 166, 6144:
-// 110 / 169 against 158 / 174, 8192: 145 / 226 against 168 / 171; FP32 2048:
-// 26 / 36 against 121 / 126, 6144: 68 / 105 against 122 / 130, 8192: 91 / 141
-// against 127 / 130.  Both give the same bits.
-constexpr int64_t coop_max_n(size_t lt) { return lt == sizeof(double) ? 6144 : 7168; }
+// latencies) until its warps fill the chip.  H2, dt = 1e-6 / 1e-4 s, ms, coop
+// against per thread: FP64 2048: 40 / 60 against 150 / 154, 6144: 110 / 169
+// against 117 / 157, 8192: 145 / 226 against 119 / 159; FP32 2048: 26 / 36
+// against 84 / 116, 6144: 68 / 105 against 86 / 118, 8192: 91 / 141 against
+// 87 / 120.  Both give the same bits.
+constexpr int64_t coop_max_n(size_t lt) { return lt == sizeof(double) ? 5632 : 6912; }
 // ... and a mechanism whose reaction tail leaves several blocks per SM
 constexpr size_t COOP_MAX_SMEM = 64 * 1024;
+
+// a finished state's status and counters, by lane 0 of its group
+template <int L>
+__device__ __forceinline__ void store_counts(const StepState &s, const KernelArgs &a, int64_t idx) {
+  if (Grp<L>::lane() != 0) return;
+  const int64_t n = a.rp.n;
+  const int32_t c[8] = {s.nstep, s.naccpt, s.nrejct, s.nfcn, s.njac, s.ndec, s.nsol, s.status};
+  if (a.status) a.status[idx] = s.status;
+  for (int q = 0; q < 8; ++q) {
+    if (a.counters) a.counters[(int64_t)q * n + idx] = c[q];
+    if (q < 7) atomicAdd(a.totals + q, (unsigned long long)c[q]);
+  }
+  if (s.status) atomicAdd(a.totals + 7, 1ull);
+  atomicMax(a.totals + 8, (unsigned long long)s.nstep);
+}
 
 // a finished state's vector, status and counters, from its group of L lanes
 template <int L>
 __device__ __forceinline__ void store_lanes(const WVecT<Grp<L>::WR> &y, const StepState &s,
                                             const KernelArgs &a, int N, int64_t idx) {
   using G = Grp<L>;
-  constexpr int WR = G::WR;
   const int lane = G::lane();
   const int64_t n = a.rp.n;
   double sum = 0.0;
 #pragma unroll
-  for (int r = 0; r < WR; ++r) {
+  for (int r = 0; r < G::WR; ++r) {
     const int g = lane + L * r;
     if (g == 0) a.T[idx] = y.v[r];
     if (g >= 1 && g < N) {
@@ -290,22 +315,8 @@ __device__ __forceinline__ void store_lanes(const WVecT<Grp<L>::WR> &y, const St
     }
   }
   sum = G::sum(sum);
-  if (lane == 0) {
-    a.Y[(int64_t)(N - 1) * n + idx] = 1.0 - sum;
-    if (a.status) a.status[idx] = s.status;
-    if (a.counters) {
-      const int32_t c[8] = {s.nstep, s.naccpt, s.nrejct, s.nfcn, s.njac, s.ndec, s.nsol,
-                            s.status};
-      for (int q = 0; q < 8; ++q) a.counters[(int64_t)q * n + idx] = c[q];
-    }
-    const unsigned long long c7[7] = {
-        (unsigned long long)s.nstep, (unsigned long long)s.naccpt, (unsigned long long)s.nrejct,
-        (unsigned long long)s.nfcn,  (unsigned long long)s.njac,   (unsigned long long)s.ndec,
-        (unsigned long long)s.nsol};
-    for (int q = 0; q < 7; ++q) atomicAdd(a.totals + q, c7[q]);
-    if (s.status) atomicAdd(a.totals + 7, 1ull);
-    atomicMax(a.totals + 8, (unsigned long long)s.nstep);
-  }
+  if (lane == 0) a.Y[(int64_t)(N - 1) * n + idx] = 1.0 - sum;
+  store_counts<L>(s, a, idx);
 }
 
 // WARP layout: one state per group of L lanes; groups pop states from the
@@ -378,11 +389,12 @@ __global__ void __launch_bounds__(TEAM_MAX *TEAM_NT, 1) k_integrate_team(KernelA
   const int N = m.ns, lane = G::lane(), warp = (int)(threadIdx.x / 32);
   const int team = warp / TEAM_WARPS, wt = warp % TEAM_WARPS;
   const int64_t n = a.rp.n;
-  const HotTables h = stage_hot(m, a.L, team_smem);  // ends with a block barrier
+  const HotTables h = stage_hot(a.L, a.hot, a.hot_smem != 0, team_smem);
   const size_t tb = team_bytes(a.L, N, sizeof(LT));
+  const size_t hb = a.hot_smem ? hot_offsets(a.L).bytes : 0;
   const int64_t slot = (int64_t)blockIdx.x * (blockDim.x / TEAM_NT) + team;  // < gslots (launch)
   const TeamBuf<LT> t = carve_team<LT>(
-      a.L, team_smem + hot_bytes(a.L) + team * tb, team, N,
+      a.L, team_smem + hb + team * tb, team, N,
       reinterpret_cast<unsigned char *>(a.gscratch) +
           slot * (int64_t)warp_slot_mats(sizeof(LT)) * N * (N + 1) * (int64_t)sizeof(LT));
   const TeamMassFrac<LT> f{m, h, t};
@@ -426,26 +438,38 @@ __global__ void __launch_bounds__(TEAM_MAX *TEAM_NT, 1) k_integrate_team(KernelA
   sys.post(TEAM_QUIT);
 }
 
-template <typename LT, bool FDJ>
-int launch_team(const KernelArgs &a, cudaStream_t st, int sms, bool &fits) {
-  if (!a.gscratch || a.gslots < 1) return KIN_ERR_UNSUPPORTED;
-  const size_t budget = 227 * 1024;
-  const size_t hot = hot_bytes(a.L), tb = team_bytes(a.L, a.L.ns, sizeof(LT));
-  // 12-bit reaction numbers and 15-bit derivative indices in the staged lists
-  fits = hot + tb <= budget && a.L.nr < 4096 && a.L.nslots + a.L.neff < 32768;
-  if (!fits) return KIN_OK;
-  int64_t teams = (int64_t)((budget - hot) / tb);
+struct TeamLaunch {
+  unsigned grid, threads;
+  size_t smem;
+};
+
+// teams per block and blocks for a batch; the tables go to shared memory when
+// a team fits beside them.  false when not even one team fits.
+inline bool team_shape(KernelArgs &a, int N, size_t lt, int sms, TeamLaunch &g) {
+  const size_t budget = 227 * 1024, tb = team_bytes(a.L, N, lt), hot = hot_offsets(a.L).bytes;
+  if (!a.hot || tb > budget) return false;
+  a.hot_smem = hot + tb <= budget;
+  const size_t fixed = a.hot_smem ? hot : 0;
+  int64_t teams = (int64_t)((budget - fixed) / tb);
   teams = teams < TEAM_MAX ? teams : TEAM_MAX;
   const int64_t want = (a.rp.n + sms - 1) / sms;  // a small batch spreads over the SMs
   teams = teams < want ? teams : want;
   int64_t grid = (a.rp.n + teams - 1) / teams;
   grid = grid < sms ? grid : sms;
-  if (grid * teams > a.gslots) grid = a.gslots / teams;
-  if (grid < 1) return KIN_ERR_UNSUPPORTED;
-  const size_t sm = hot + teams * tb;
+  if (grid * teams > a.gslots) grid = a.gslots / teams;  // one slot per team
+  if (grid < 1) return false;
+  g = TeamLaunch{(unsigned)grid, (unsigned)(teams * TEAM_NT), fixed + teams * tb};
+  return true;
+}
+
+template <typename LT, bool FDJ>
+int launch_team(KernelArgs a, cudaStream_t st, int sms) {
+  if (!a.gscratch || a.gslots < 1) return KIN_ERR_UNSUPPORTED;
+  TeamLaunch g;
+  if (!team_shape(a, a.L.ns, sizeof(LT), sms, g)) return KIN_ERR_UNSUPPORTED;
   auto kern = k_integrate_team<LT, FDJ>;
-  KIN_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
-  kern<<<(unsigned)grid, (unsigned)(teams * TEAM_NT), sm, st>>>(a);
+  KIN_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g.smem));
+  kern<<<g.grid, g.threads, g.smem, st>>>(a);
   KIN_CUDA_TRY(cudaGetLastError());
   return KIN_OK;
 }
@@ -489,15 +513,12 @@ int launch_t(const KernelArgs &a, const kin_options &o, cudaStream_t st, int sms
   if (o.layout == KIN_LAYOUT_WARP) {
     if constexpr (MAXN == 64) {
       if (a.L.ns > 63) return KIN_ERR_UNSUPPORTED;
-      bool fits = false;
-      const int rc = launch_team<LT, FDJ>(a, st, sms, fits);
-      if (fits) return rc;
-      // more reactions than a team's shared memory holds: a state per thread
+      return launch_team<LT, FDJ>(a, st, sms);
     } else {
       return KIN_ERR_UNSUPPORTED;
     }
   }
-  const bool plain = o.layout != KIN_LAYOUT_QUEUE;
+  const bool plain = o.layout == KIN_LAYOUT_PLAIN;
   const int block = o.block > 0 ? o.block : 64;
   if (block > 64 || block % 32) return KIN_ERR_INVALID_ARG;
   const size_t sm = thread_smem_bytes<MAXN>(a.L, block);
@@ -514,7 +535,16 @@ int launch_t(const KernelArgs &a, const kin_options &o, cudaStream_t st, int sms
     }
   }
   if (plain) {
-    auto kern = k_integrate_plain<MAXN, LT, FDJ>;
+    void (*kern)(KernelArgs) = k_integrate_plain<MAXN, LT, FDJ, KIN_THREAD_MIN_BLOCKS>;
+    if constexpr (MAXN <= 16 && !FDJ) {
+      const int64_t per_sm = (a.rp.n + 64ll * sms - 1) / (64ll * sms);
+      if (per_sm <= PLAIN_BLOCKS_FEW)
+        kern = k_integrate_plain<MAXN, LT, FDJ, PLAIN_BLOCKS_FEW>;
+      else if (per_sm <= PLAIN_BLOCKS_MID)
+        kern = k_integrate_plain<MAXN, LT, FDJ, PLAIN_BLOCKS_MID>;
+      else if (per_sm <= PLAIN_BLOCKS_MANY)
+        kern = k_integrate_plain<MAXN, LT, FDJ, PLAIN_BLOCKS_MANY>;
+    }
     KIN_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
     KIN_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, carve));
     const int64_t grid = (a.rp.n + block - 1) / block;

@@ -129,5 +129,7 @@ extern "C" int kin_integrate_static(const kin_mech_desc *desc, double *Y, double
   a.order = nullptr;
   a.gscratch = nullptr;  // the thread layout needs no group slots
   a.gslots = 0;
+  a.hot = nullptr;
+  a.hot_smem = 0;
   return launch_dispatch(a, o, st, sms);
 }

@@ -73,139 +73,68 @@ struct HotTables {
   const unsigned short *term;  // index << 1 | (1 for a reactant's row: minus)
 };
 
-__device__ __forceinline__ int rec_type(uint2 r) { return (r.x >> 24) & 3; }
-__device__ __forceinline__ int rec_nre(uint2 r) { return (r.x >> 26) & 3; }
-__device__ __forceinline__ int rec_npr(uint2 r) { return (r.x >> 28) & 3; }
+__host__ __device__ __forceinline__ int rec_type(uint2 r) { return (r.x >> 24) & 3; }
+__host__ __device__ __forceinline__ int rec_nre(uint2 r) { return (r.x >> 26) & 3; }
+__host__ __device__ __forceinline__ int rec_npr(uint2 r) { return (r.x >> 28) & 3; }
 // species in slot s: reactants 0-2, products 3-5
-__device__ __forceinline__ int rec_slot(uint2 r, int s) {
+__host__ __device__ __forceinline__ int rec_slot(uint2 r, int s) {
   return s < 3 ? (int)(r.x >> (8 * s)) & 255 : (int)(r.y >> (8 * (s - 3))) & 255;
 }
 
-// round of 32 reactions, and position of the slot among the reaction's
-__device__ __forceinline__ int group_key(const uint2 *rec, int code) {
-  const int slot = code & 7;
-  return (code >> 8) << 3 | (slot < 3 ? slot : slot - 3 + rec_nre(rec[code >> 3]));
+// Where the tables lie in their buffer (byte offsets), which the host fills
+// once per mechanism (build_hot) and a block copies to shared memory.
+struct HotOffsets {
+  size_t d, rec, ints, net, occ, off, term, rank, col, bytes;
+};
+__host__ __device__ inline HotOffsets hot_offsets(const MechLayout &L) {
+  HotOffsets o;
+  const size_t nr = L.nr, ns = L.ns, ncsr = L.ni - L.icsr;
+  o.d = 0;
+  o.rec = sizeof(double) * (4 * nr + EXP_TAB);
+  o.ints = o.rec + sizeof(uint2) * nr;
+  o.net = o.ints + sizeof(int) * 3 * (ns + 2);
+  o.occ = o.net + 2 * ncsr;
+  o.off = o.occ + 2 * (size_t)L.nslots;
+  o.term = o.off + 2 * nr;
+  o.rank = o.term + 2 * (size_t)L.nterms;
+  o.col = o.rank + 64;
+  o.bytes = (o.col + L.nslots + L.neff + 15) / 16 * 16;
+  return o;
 }
 
-__host__ __device__ inline size_t hot_bytes(const MechLayout &L) {
-  const int ns = L.ns, nr = L.nr, ncsr = L.ni - L.icsr;
-  size_t b = sizeof(double) * (4 * (size_t)nr + EXP_TAB) + sizeof(uint2) * (size_t)nr;
-  b += sizeof(int) * 3 * (size_t)(ns + 2);
-  b += sizeof(unsigned short) * ((size_t)L.nslots + ncsr + nr + L.nterms);
-  b += 64 + (size_t)L.nslots + L.neff;
-  return (b + 15) / 16 * 16;
+__device__ __forceinline__ HotTables hot_view(const MechLayout &L, const unsigned char *p) {
+  const HotOffsets o = hot_offsets(L);
+  const double *d = reinterpret_cast<const double *>(p);
+  const int nr = L.nr, *ints = reinterpret_cast<const int *>(p + o.ints);
+  HotTables h;
+  h.lnA = d;
+  h.b = d + nr;
+  h.Th = d + 2 * nr;
+  h.dnu = d + 3 * nr;
+  h.etab = d + 4 * nr;
+  h.rec = reinterpret_cast<const uint2 *>(p + o.rec);
+  h.net0 = ints;
+  h.occ0 = ints + L.ns + 2;
+  h.term0 = ints + 2 * (L.ns + 2);
+  h.net = reinterpret_cast<const unsigned short *>(p + o.net);
+  h.occ = reinterpret_cast<const unsigned short *>(p + o.occ);
+  h.off = reinterpret_cast<const unsigned short *>(p + o.off);
+  h.term = reinterpret_cast<const unsigned short *>(p + o.term);
+  h.rank = p + o.rank;
+  h.col = p + o.col;
+  return h;
 }
 
-__device__ inline HotTables stage_hot(const MechView &m, const MechLayout &L, unsigned char *smem) {
-  const int nt = blockDim.x, tid = threadIdx.x, nr = m.nr, ns = m.ns, ncsr = L.ni - L.icsr;
-  const int nslots = L.nslots;
-  double *d = reinterpret_cast<double *>(smem);
-  double *lnA = d, *b = d + nr, *Th = d + 2 * nr, *dnu = d + 3 * nr, *et = d + 4 * nr;
-  uint2 *rec = reinterpret_cast<uint2 *>(et + EXP_TAB);
-  int *net0 = reinterpret_cast<int *>(rec + nr), *occ0 = net0 + ns + 2, *term0 = occ0 + ns + 2;
-  unsigned short *net = reinterpret_cast<unsigned short *>(term0 + ns + 2), *occ = net + ncsr;
-  unsigned short *off = occ + nslots, *term = off + nr;
-  unsigned char *rank = reinterpret_cast<unsigned char *>(term + L.nterms), *col = rank + 64;
-  for (int i = tid; i < nr; i += nt) {
-    lnA[i] = m.lnA[i];
-    b[i] = m.b[i];
-    Th[i] = m.Th[i];
-    dnu[i] = m.dnu[i];
-    const int meta = m.meta[i];
-    const int *sl = m.slot + 6 * i;
-    uint2 r = {(unsigned)(meta & 63) << 24, 0u};
-    for (int s = 0; s < meta_nreac(meta); ++s) r.x |= (unsigned)sl[s] << (8 * s);
-    for (int s = 0; s < meta_nprod(meta); ++s) r.y |= (unsigned)sl[3 + s] << (8 * s);
-    rec[i] = r;
-  }
-  for (int j = tid; j < EXP_TAB; j += nt) et[j] = m.etab[j];
-  for (int k = tid; k <= ns; k += nt) net0[k] = m.csr0[k];
-  for (int e = tid; e < ncsr; e += nt) net[e] = (unsigned short)m.csr[e];
+// the block's copy in shared memory, or the tables where they are when a
+// mechanism's lists leave no room for a team beside them; whole block
+__device__ __forceinline__ HotTables stage_hot(const MechLayout &L, const unsigned char *hot,
+                                               bool copy, unsigned char *smem) {
+  if (!copy) return hot_view(L, hot);
+  const uint4 *src = reinterpret_cast<const uint4 *>(hot);
+  uint4 *dst = reinterpret_cast<uint4 *>(smem);
+  for (size_t e = threadIdx.x; e < hot_offsets(L).bytes / 16; e += blockDim.x) dst[e] = src[e];
   __syncthreads();
-  for (int pass = 0; pass < 2; ++pass) {
-    if (tid < ns) {
-      int cnt = 0;
-      for (int i0 = 0; i0 < nr; i0 += 32)
-        for (int rs = 0; rs < 6; ++rs)
-#pragma unroll 1
-          for (int i = i0; i < i0 + 32 && i < nr; ++i) {
-            const uint2 r = rec[i];
-            const int nre = rec_nre(r), npr = rec_npr(r);
-            const int slot = rs < nre ? rs : rs < nre + npr ? 3 + rs - nre : -1;
-            if (slot < 0 || rec_slot(r, slot) != tid) continue;
-            if (pass) occ[occ0[tid] + cnt] = (unsigned short)(i << 3 | slot);
-            ++cnt;
-          }
-      if (!pass) occ0[tid + 1] = cnt;
-    }
-    __syncthreads();
-    if (!pass && tid == 0) {
-      occ0[0] = 0;
-      for (int k = 0; k < ns; ++k) occ0[k + 1] += occ0[k];
-    }
-    __syncthreads();
-  }
-  if (tid < ns - 1) {
-    const int mine = occ0[tid + 1] - occ0[tid];
-    int r = 0;
-    for (int k = 0; k < ns - 1; ++k) {
-      const int o = occ0[k + 1] - occ0[k];
-      r += o > mine || (o == mine && k < tid);
-    }
-    rank[r] = (unsigned char)tid;
-  }
-  if (tid == 0) {
-    int o = 0;
-    for (int i = 0; i < nr; ++i) {
-      off[i] = (unsigned short)o;
-      o += rec_nre(rec[i]) + rec_npr(rec[i]);
-    }
-  }
-  __syncthreads();
-  for (int i = tid; i < nr; i += nt) {
-    const uint2 r = rec[i];
-    const int nre = rec_nre(r), npr = rec_npr(r);
-    for (int s = 0; s < nre + npr; ++s)
-      col[off[i] + s] = (unsigned char)rec_slot(r, s < nre ? s : 3 + s - nre);
-  }
-  for (int e = tid; e < L.neff; e += nt) col[nslots + e] = (unsigned char)m.effsp[e];
-  // a row's terms: per round of 32 reactions and slot position, first the
-  // slots' derivatives (position by position over the group's reactions), then
-  // the collision partners'
-  for (int pass = 0; pass < 2; ++pass) {
-    if (tid < ns) {
-      int cnt = 0;
-      const int o1 = occ0[tid + 1];
-      for (int o = occ0[tid], oe; o < o1; o = oe) {
-        const int key = group_key(rec, occ[o]);
-        int ne = 0;
-        for (oe = o; oe < o1 && group_key(rec, occ[oe]) == key; ++oe)
-          ne = max(ne, (occ[oe] >> 3) < m.nfall ? meta_neff(m.meta[occ[oe] >> 3]) : 0);
-        for (int x = 0; x < 6 + ne; ++x)
-#pragma unroll 1
-          for (int q = o; q < oe; ++q) {
-            const int i = occ[q] >> 3, neg = (occ[q] & 7) < 3;
-            const int nsl = rec_nre(rec[i]) + rec_npr(rec[i]);
-            int idx = -1;
-            if (x < 6)
-              idx = x < nsl ? off[i] + x : -1;
-            else if (i < m.nfall && x - 6 < meta_neff(m.meta[i]))
-              idx = nslots + m.eff0[i] + x - 6;
-            if (idx < 0) continue;
-            if (pass) term[term0[tid] + cnt] = (unsigned short)(idx << 1 | neg);
-            ++cnt;
-          }
-      }
-      if (!pass) term0[tid + 1] = cnt;
-    }
-    __syncthreads();
-    if (!pass && tid == 0) {
-      term0[0] = 0;
-      for (int k = 0; k < ns; ++k) term0[k + 1] += term0[k];
-    }
-    __syncthreads();
-  }
-  return HotTables{lnA, b, Th, dnu, et, rec, net0, occ0, net, occ, rank, off, col, term0, term};
+  return hot_view(L, smem);
 }
 
 // ---------------------------------------------------------------------------
@@ -225,7 +154,8 @@ struct TeamBuf {
   double *Jd;        // the FP64 assembly matrix, over E2
   double *w0, *w12;  // warp 0's C, g, q; warp 1's, then warp 2's
   double *js;        // Jacobian scratch, over E1 and warp 1's and 2's buffers
-  LT *dr, *dd;       // E2's pivots: Smith's ratio and denominator
+  LT *dr, *dd, *di;  // E2's pivots: Smith's ratio, denominator and its reciprocal
+  LT *d1;            // reciprocals of E1's pivots (FP64)
   unsigned char *p1, *p2;  // row sources after all exchanges (p2: bit 7 Smith's case)
   TeamCtl *ctl;
   __device__ __forceinline__ double *C(int w) const { return w ? w12 + (w - 1) * wstride : w0; }
@@ -249,7 +179,7 @@ __host__ __device__ inline size_t team_bytes(const MechLayout &L, int N, size_t 
   if (need > mid) mid = need;
   size_t b = (sizeof(TeamCtl) + 15) / 16 * 16 + w + mid;
   if (!warp_e2_global(lt)) b += 2 * mat * lt;
-  b += 2 * (size_t)team_nv(N) * lt + 128;
+  b += 4 * (size_t)team_nv(N) * lt + 128;
   return (b + 15) / 16 * 16;
 }
 
@@ -284,7 +214,9 @@ __device__ TeamBuf<LT> carve_team(const MechLayout &L, unsigned char *p, int tea
   p += e1 + w2 > need ? e1 + w2 : need;
   t.dr = reinterpret_cast<LT *>(p);
   t.dd = t.dr + team_nv(N);
-  p += 2 * (size_t)team_nv(N) * sizeof(LT);
+  t.di = t.dr + 2 * team_nv(N);
+  t.d1 = t.dr + 3 * team_nv(N);
+  p += 4 * (size_t)team_nv(N) * sizeof(LT);
   t.p1 = p;
   t.p2 = p + 64;
   return t;
@@ -298,9 +230,6 @@ __device__ __forceinline__ void named_sync(int id, int nt) {
 // ---------------------------------------------------------------------------
 // Rates
 // ---------------------------------------------------------------------------
-#ifndef KC_FIRST
-#define KC_FIRST(a, b, c) t_fma(a, b, -(c))
-#endif
 // ln Kc's and the products' sums over a reaction's slots, in slot order
 struct SlotSums {
   double fwd, rev, lnKc;
@@ -308,7 +237,7 @@ struct SlotSums {
 __device__ __forceinline__ SlotSums slot_sums(const HotTables &h, const double *C, const double *g,
                                               int i, uint2 r, double lnPf) {
   const int nre = rec_nre(r), npr = rec_npr(r);
-  SlotSums o = {1.0, 1.0, KC_FIRST(h.dnu[i], lnPf, g[r.x & 255])};
+  SlotSums o = {1.0, 1.0, t_fma(h.dnu[i], lnPf, -g[r.x & 255])};
   o.fwd = C[r.x & 255];
   o.rev = C[r.y & 255];
   if (nre > 1) {
@@ -456,11 +385,48 @@ __device__ __noinline__ int team_rhs(const MechView &m, const HotTables &h, doub
   return G::all(ok) ? 0 : 4;
 }
 
+__device__ __forceinline__ double flip(double x, int sign) {
+  return __hiloint2double(__double2hiint(x) ^ sign, __double2loint(x));
+}
+
+// sums over species k's reactions of nu sig and nu dq/dT
+__device__ __forceinline__ void row_sums(const HotTables &h, const double *sig, const double *dq,
+                                         int k, double &b, double &tc) {
+#pragma unroll 2
+  for (int o = h.occ0[k]; o < h.occ0[k + 1]; ++o) {
+    const int code = h.occ[o], i = code >> 3, neg = (code & 7) < 3 ? 0x80000000 : 0;
+    b += flip(sig[i], neg);
+    tc += flip(dq[i], neg);
+  }
+}
+
+// species k's sparse Jacobian row: its terms added to Jr[column], or to a for
+// the inert's; the next term's operands are loaded before this one's store
+__device__ __forceinline__ void row_terms(const HotTables &h, const double *D, int k, int inert,
+                                          double *Jr, double &a) {
+  const int e1 = h.term0[k + 1];
+  int x = h.term0[k];
+  int code = x < e1 ? h.term[x] : 0, col = h.col[code >> 1];
+  double d = D[code >> 1];
+#pragma unroll 1
+  for (; x < e1; ++x) {
+    const int c0 = col, neg = code << 31;
+    const double v = flip(d, neg);
+    code = x + 1 < e1 ? h.term[x + 1] : 0;
+    col = h.col[code >> 1];
+    d = D[code >> 1];
+    if (c0 != inert)
+      Jr[c0] += v;
+    else
+      a += v;
+  }
+}
+
 // One reaction with what its Jacobian terms need: the net rate, the forward
 // and (negated) reverse rate constants with the falloff factor, dq/dM,
-// sum_l C_l dq/dC_l and dq/dT at fixed Y.
+// sum_l C_l dq/dC_l, dq/dT at fixed Y, and dq/dT at fixed moles and volume.
 struct ReactionJac {
-  double q, pkf, pkr, u, sig, dqdT;
+  double q, pkf, pkr, u, sig, dqdT, dqdT_nV;
 };
 __device__ __forceinline__ ReactionJac reaction_jac(const MechView &m, const HotTables &h,
                                                     const double *C, const double *g,
@@ -510,6 +476,7 @@ __device__ __forceinline__ ReactionJac reaction_jac(const MechView &m, const Hot
   r.sig = phi * (nre * kf * fwd - npr * kr * rev) + r.u * (M - Ctot);
   r.dqdT = phi * (kf * dlnkf * fwd - kr * dlnkr * rev) + Rn * dphi_dT -
            (r.sig + r.u * Ctot) * invT;
+  r.dqdT_nV = phi * (kf * dlnkf * fwd - kr * dlnkr * rev) + Rn * dphi_dT - r.u * Ctot * invT;
   r.pkf = phi * kf;
   r.pkr = -phi * kr;
   return r;
@@ -557,9 +524,10 @@ __device__ __forceinline__ void row_set(X &a, X &b, int i, X v) {
   if ((int)(threadIdx.x & 31) == (i & 31)) (i < 32 ? a : b) = v;
 }
 
-// Real LU with partial pivoting on one warp; returns 0 or k + 1.
-template <typename LT>
-__device__ __noinline__ int team_lu_real(int N, int ld, LT *a, unsigned char *perm) {
+// Real LU on one warp, with partial pivoting or (PIVOT false) in the given
+// order; returns 0 or k + 1.
+template <typename LT, bool PIVOT>
+__device__ __noinline__ int team_lu_real(int N, int ld, LT *a, unsigned char *perm, LT *d1) {
   const int lane = threadIdx.x & 31;
   int src0 = lane, src1 = lane + 32;
   for (int kb = 0; kb < N; kb += TEAM_PANEL) {
@@ -575,21 +543,32 @@ __device__ __noinline__ int team_lu_real(int N, int ld, LT *a, unsigned char *pe
     __syncwarp();
 #pragma unroll 1
     for (int c = 0; c < nb; ++c) {
-      const int k = kb + c, p = arg_pivot(fabs(p0[0]), fabs(p1[0]), k, N);
-      if (p < 0) return k + 1;
+      const int k = kb + c;
+      int p = k;
+      if constexpr (PIVOT) {
+        p = arg_pivot(fabs(p0[0]), fabs(p1[0]), k, N);
+        if (p < 0) return k + 1;
+      } else if (!(fabs(row_get(p0[0], p1[0], k)) > LT(0))) {
+        return k + 1;
+      }
       pivs |= (unsigned)p << (8 * c);
       LT rp[TEAM_PANEL];
 #pragma unroll
       for (int d = 0; d < TEAM_PANEL; ++d) {
-        const LT vk = row_get(p0[d], p1[d], k);
         rp[d] = row_get(p0[d], p1[d], p);
-        row_set(p0[d], p1[d], p, vk);
-        row_set(p0[d], p1[d], k, rp[d]);
+        if constexpr (PIVOT) {
+          const LT vk = row_get(p0[d], p1[d], k);
+          row_set(p0[d], p1[d], p, vk);
+          row_set(p0[d], p1[d], k, rp[d]);
+        }
       }
-      const int sk = row_get(src0, src1, k), sp = row_get(src0, src1, p);
-      row_set(src0, src1, p, sk);
-      row_set(src0, src1, k, sp);
+      if constexpr (PIVOT) {
+        const int sk = row_get(src0, src1, k), sp = row_get(src0, src1, p);
+        row_set(src0, src1, p, sk);
+        row_set(src0, src1, k, sp);
+      }
       const LT inv = LT(1) / rp[0];
+      if (lane == 0) d1[k] = inv;
       const bool on0 = lane > k && lane < N, on1 = lane + 32 > k && lane + 32 < N;
       if (on0) p0[0] = t_mul(p0[0], inv);
       if (on1) p1[0] = t_mul(p1[0], inv);
@@ -664,6 +643,21 @@ __device__ __noinline__ int team_lu_real(int N, int ld, LT *a, unsigned char *pe
   return 0;
 }
 
+// a / d.  FP32 divides.  FP64, where an IEEE division costs nine instructions
+// of the bounding pipe, corrects a times the reciprocal r = 1/d once with the
+// exact residual (Markstein, IBM J. Res. Dev. 34, 1990): at most the last bit
+// away from the rounded quotient.  A quotient outside the normal range is left
+// to the division.
+__device__ __forceinline__ float quot(float a, float d, float) { return a / d; }
+__device__ __forceinline__ double quot(double a, double d, double r) {
+  const double q = a * r;
+  const int e = (__double2hiint(q) >> 20) & 0x7ff, f = (__double2hiint(a) >> 20) & 0x7ff;
+  if (e < 64 || e > 1980 || f < 64) return a / d;
+  return t_fma(t_fma(-q, d, a), r, q);
+}
+__device__ __forceinline__ float recip(float) { return 0.0f; }  // unused: FP32 divides
+__device__ __forceinline__ double recip(double d) { return 1.0 / d; }
+
 // ratio and denominator of Smith's complex division by re + i im (cdiv)
 template <typename LT>
 __device__ __forceinline__ int smith_div(LT re, LT im, LT &r, LT &den) {
@@ -677,14 +671,15 @@ __device__ __forceinline__ int smith_div(LT re, LT im, LT &r, LT &den) {
   return 1;
 }
 template <typename LT>
-__device__ __forceinline__ void smith_quot(LT a, LT b, LT r, LT den, int mode, LT &re, LT &im) {
-  re = (mode ? t_fma(a, r, b) : t_fma(b, r, a)) / den;
-  im = (mode ? t_fma(b, r, -a) : t_fma(-a, r, b)) / den;
+__device__ __forceinline__ void smith_quot(LT a, LT b, LT r, LT den, LT iden, int mode, LT &re,
+                                           LT &im) {
+  re = quot(mode ? t_fma(a, r, b) : t_fma(b, r, a), den, iden);
+  im = quot(mode ? t_fma(b, r, -a) : t_fma(-a, r, b), den, iden);
 }
 
 // Complex LU on warps 1 and 2 of a team: warp 1 factorises the panel, both
 // update the rest, a column per lane.
-template <typename LT>
+template <typename LT, bool PIVOT>
 __device__ __noinline__ int team_lu_cplx(int N, const TeamBuf<LT> &t, int wt) {
   const int lane = threadIdx.x & 31, ld = t.ld, col = lane + 32 * (wt - 1), bar = t.bar + TEAM_MAX;
   cplx_t<LT> *a = t.E2;
@@ -705,8 +700,12 @@ __device__ __noinline__ int team_lu_cplx(int N, const TeamBuf<LT> &t, int wt) {
       __syncwarp();
 #pragma unroll 1
       for (int c = 0; c < nb; ++c) {
-        const int k = kb + c, p = arg_pivot(fabs(p0[0].x) + fabs(p0[0].y),
-                                            fabs(p1[0].x) + fabs(p1[0].y), k, N);
+        const int k = kb + c;
+        int p = k;
+        if constexpr (PIVOT)
+          p = arg_pivot(fabs(p0[0].x) + fabs(p0[0].y), fabs(p1[0].x) + fabs(p1[0].y), k, N);
+        else if (!(row_get(fabs(p0[0].x) + fabs(p0[0].y), fabs(p1[0].x) + fabs(p1[0].y), k) > LT(0)))
+          p = -1;
         if (p < 0) {
           sing = k + 1;
           break;
@@ -715,17 +714,21 @@ __device__ __noinline__ int team_lu_cplx(int N, const TeamBuf<LT> &t, int wt) {
         cplx_t<LT> rp[TEAM_PANEL];
 #pragma unroll
         for (int d = 0; d < TEAM_PANEL; ++d) {
-          const LT xk = row_get(p0[d].x, p1[d].x, k), yk = row_get(p0[d].y, p1[d].y, k);
           rp[d].x = row_get(p0[d].x, p1[d].x, p);
           rp[d].y = row_get(p0[d].y, p1[d].y, p);
-          row_set(p0[d].x, p1[d].x, p, xk);
-          row_set(p0[d].y, p1[d].y, p, yk);
-          row_set(p0[d].x, p1[d].x, k, rp[d].x);
-          row_set(p0[d].y, p1[d].y, k, rp[d].y);
+          if constexpr (PIVOT) {
+            const LT xk = row_get(p0[d].x, p1[d].x, k), yk = row_get(p0[d].y, p1[d].y, k);
+            row_set(p0[d].x, p1[d].x, p, xk);
+            row_set(p0[d].y, p1[d].y, p, yk);
+            row_set(p0[d].x, p1[d].x, k, rp[d].x);
+            row_set(p0[d].y, p1[d].y, k, rp[d].y);
+          }
         }
-        const int sk = row_get(src0, src1, k), sp = row_get(src0, src1, p);
-        row_set(src0, src1, p, sk);
-        row_set(src0, src1, k, sp);
+        if constexpr (PIVOT) {
+          const int sk = row_get(src0, src1, k), sp = row_get(src0, src1, p);
+          row_set(src0, src1, p, sk);
+          row_set(src0, src1, k, sp);
+        }
         LT r, den;
         const unsigned mode = smith_div(rp[0].x, rp[0].y, r, den);
         if (lane == 0) {
@@ -734,8 +737,10 @@ __device__ __noinline__ int team_lu_cplx(int N, const TeamBuf<LT> &t, int wt) {
         }
         row_set(mode0, mode1, k, mode);
         const bool on0 = lane > k && lane < N, on1 = lane + 32 > k && lane + 32 < N;
-        if (on0) smith_quot(p0[0].x, p0[0].y, r, den, (int)mode, p0[0].x, p0[0].y);
-        if (on1) smith_quot(p1[0].x, p1[0].y, r, den, (int)mode, p1[0].x, p1[0].y);
+        const LT iden = recip(den);
+        if (lane == 0) t.di[k] = iden;
+        if (on0) smith_quot(p0[0].x, p0[0].y, r, den, iden, (int)mode, p0[0].x, p0[0].y);
+        if (on1) smith_quot(p1[0].x, p1[0].y, r, den, iden, (int)mode, p1[0].x, p1[0].y);
         if (lane < c && p != k) {  // the finished columns of the panel
           const cplx_t<LT> x = a[k * ld + kb + lane];
           a[k * ld + kb + lane] = a[p * ld + kb + lane];
@@ -765,19 +770,26 @@ __device__ __noinline__ int team_lu_cplx(int N, const TeamBuf<LT> &t, int wt) {
 #pragma unroll
     for (int c = 0; c < TEAM_PANEL; ++c) piv[c] = t.ctl->piv[c];
     const int jt = kb + nb;
+    // more than 32 columns left: a column per lane of both warps.  Fewer: both
+    // warps have the same columns and halve the rows; warp 1 exchanges and
+    // forms U there while warp 2 exchanges the finished columns.
+    // (FP32 keeps its columns: the second barrier cost more than the rows gave)
+    constexpr int UNROLL = sizeof(LT) == 4 ? 1 : 2;
+    const bool wide = sizeof(LT) == 4 || N - jt > 32;
+    if (wide || wt == 2)
 #pragma unroll 1
-    for (int j = col; j < kb; j += 64)
+      for (int j = wide ? col : lane; j < kb; j += wide ? 64 : 32)
 #pragma unroll
-      for (int c = 0; c < TEAM_PANEL; ++c)
-        if (piv[c] != kb + c) {
-          const cplx_t<LT> x = a[(kb + c) * ld + j];
-          a[(kb + c) * ld + j] = a[piv[c] * ld + j];
-          a[piv[c] * ld + j] = x;
-        }
-#pragma unroll 1
-    for (int j = jt + col; j < N; j += 64) {
-      cplx_t<LT> u[TEAM_PANEL];
-      bool nz[TEAM_PANEL];
+        for (int c = 0; c < TEAM_PANEL; ++c)
+          if (piv[c] != kb + c) {
+            const cplx_t<LT> x = a[(kb + c) * ld + j];
+            a[(kb + c) * ld + j] = a[piv[c] * ld + j];
+            a[piv[c] * ld + j] = x;
+          }
+    const int j = jt + (wide ? col : lane);
+    cplx_t<LT> u[TEAM_PANEL];
+    bool nz[TEAM_PANEL];
+    if (j < N && (wide || wt == 1)) {  // only full panels have columns to the right
 #pragma unroll
       for (int c = 0; c < TEAM_PANEL; ++c) {
         const cplx_t<LT> x = a[piv[c] * ld + j];
@@ -796,8 +808,19 @@ __device__ __noinline__ int team_lu_cplx(int N, const TeamBuf<LT> &t, int wt) {
         nz[c] = u[c].x != LT(0) || u[c].y != LT(0);
         if (c) a[(kb + c) * ld + j] = u[c];
       }
-#pragma unroll 1
-      for (int i = jt; i < N; ++i) {
+    }
+    if (!wide) {
+      named_sync(bar, 64);
+      if (wt == 2 && j < N)
+#pragma unroll
+        for (int c = 0; c < TEAM_PANEL; ++c) {
+          u[c] = a[(kb + c) * ld + j];
+          nz[c] = u[c].x != LT(0) || u[c].y != LT(0);
+        }
+    }
+    if (j < N) {
+#pragma unroll UNROLL
+      for (int i = wide ? jt : jt + wt - 1; i < N; i += wide ? 1 : 2) {
         cplx_t<LT> v = a[i * ld + j];
         const cplx_t<LT> *l = a + i * ld + kb;
 #pragma unroll
@@ -820,7 +843,7 @@ __device__ __noinline__ int team_lu_cplx(int N, const TeamBuf<LT> &t, int wt) {
 // ---------------------------------------------------------------------------
 template <typename LT>
 __device__ __noinline__ void team_solve_real(int N, int ld, const LT *lu, const unsigned char *perm,
-                                             WVecT<2> &x) {
+                                             const LT *d1, WVecT<2> &x) {
   const int lane = threadIdx.x & 31, i1 = lane + 32;
   const unsigned FULL = 0xffffffffu;
   const int q0 = lane < N ? perm[lane] : 0, q1 = i1 < N ? perm[i1] : 0;
@@ -843,14 +866,14 @@ __device__ __noinline__ void team_solve_real(int N, int ld, const LT *lu, const 
   }
 #pragma unroll 1
   for (int i = N - 1; i >= 32; --i) {  // backward
-    const LT xi = __shfl_sync(FULL, v1, i - 32) / lu[i * ld + i];
+    const LT xi = quot(__shfl_sync(FULL, v1, i - 32), lu[i * ld + i], d1[i]);
     if (i1 == i) v1 = xi;
     if (i1 < i) v1 = t_fma(-r1[i], xi, v1);
     v0 = t_fma(-r0[i], xi, v0);
   }
 #pragma unroll 1
   for (int i = n0 - 1; i >= 0; --i) {
-    const LT xi = __shfl_sync(FULL, v0, i) / lu[i * ld + i];
+    const LT xi = quot(__shfl_sync(FULL, v0, i), lu[i * ld + i], d1[i]);
     if (lane == i) v0 = xi;
     if (lane < i) v0 = t_fma(-r0[i], xi, v0);
   }
@@ -903,7 +926,7 @@ __device__ __noinline__ void team_solve_cplx(int N, const TeamBuf<LT> &t, WVecT<
     const LT a = i >= 32 ? __shfl_sync(FULL, r1, i - 32) : __shfl_sync(FULL, r0, i);
     const LT b = i >= 32 ? __shfl_sync(FULL, m1, i - 32) : __shfl_sync(FULL, m0, i);
     LT qr, qi;
-    smith_quot(a, b, t.dr[i], t.dd[i], t.p2[i] >> 7, qr, qi);
+    smith_quot(a, b, t.dr[i], t.dd[i], t.di[i], t.p2[i] >> 7, qr, qi);
     if (lane == i) {
       r0 = qr;
       m0 = qi;
@@ -946,6 +969,7 @@ __device__ __forceinline__ void vec_load(int N, const double *p, WVecT<2> &x) {
 // The mass-fraction reactor on a team.
 template <typename LT>
 struct TeamMassFrac {
+  static constexpr bool PIVOT = true;
   const MechView &m;
   const HotTables &h;
   const TeamBuf<LT> &t;
@@ -1022,6 +1046,16 @@ struct TeamMassFrac {
 
   // The right-hand side (into warp 0's g buffer) and the Jacobian (into J).
   __device__ __noinline__ void jac(int wt) const {
+    LT *J = t.J;
+    const int ld = t.ld;
+    jac_out<TEAM_WARPS>(wt, [J, ld](int i, int c, double v) { J[(size_t)c * ld + i] = LT(v); });
+  }
+
+  // the same on TW warps (one: all phases on one warp, no team barrier), with
+  // the Jacobian's entries given to put(i, j, value)
+  template <int TW, class Put>
+  __device__ __forceinline__ void jac_out(int wt, Put put) const {
+    constexpr int NT = 32 * TW;
     using G = Grp<32>;
     const int lane = G::lane(), ns = m.ns, in = ns - 1, N = ns, nv = t.nv, nr = m.nr, ld = t.ld;
     TeamCtl &ct = *t.ctl;
@@ -1032,10 +1066,10 @@ struct TeamMassFrac {
     const double T = ct.T, logT = ct.logT, invT = ct.invT, rho = ct.rho, S = ct.S;
     const double Ctot = rho * S, *C = t.C(0), *g = t.g(0);
     double *q = t.q(0);
-    for (int e = lane + 32 * wt; e < N * ld; e += TEAM_NT) t.Jd[e] = 0.0;
+    for (int e = lane + 32 * wt; e < N * ld; e += NT) t.Jd[e] = 0.0;
     // reactions in rounds of 32, dealt over the warps (the Troe rounds first)
 #pragma unroll 1
-    for (int i = lane + 32 * wt; i < nr; i += TEAM_NT) {
+    for (int i = lane + 32 * wt; i < nr; i += NT) {
       const ReactionJac r = reaction_jac(m, h, C, g, hs, i, T, logT, invT, Ctot);
       q[i] = r.q;
       sig[i] = r.sig;
@@ -1064,7 +1098,7 @@ struct TeamMassFrac {
         }
       }
     }
-    named_sync(t.bar, TEAM_NT);
+    jac_sync<TW>();
     if (wt == 0) {
       // production rates and f
       WVecT<2> f;
@@ -1097,56 +1131,35 @@ struct TeamMassFrac {
         ct.CPw = cpw;
         if (!ok) ct.ret[0] = 4;
       }
-    } else {
+    }
+    if (TW == 1 || wt != 0) {
       // sparse rows of dwdot/dY, the longest lists on warp 1
-      for (int e = lane + 32 * (wt - 1); e < in; e += 64) {
+      for (int e = lane + (TW == 1 ? 0 : 32 * (wt - 1)); e < in; e += TW == 1 ? 32 : 64) {
         const int k = h.rank[e];
         double *Jr = t.Jd + (1 + k) * ld;
         double a = 0.0, b = 0.0, tc = 0.0;
-#pragma unroll 2
-        for (int o = h.occ0[k]; o < h.occ0[k + 1]; ++o) {
-          const int code = h.occ[o], i = code >> 3, neg = (code & 7) < 3 ? 0x80000000 : 0;
-          b += flip(sig[i], neg);
-          tc += flip(dq[i], neg);
-        }
-        // the next term's operands are loaded before this one's store
-        const int e1 = h.term0[k + 1];
-        int x = h.term0[k];
-        int code = x < e1 ? h.term[x] : 0, col = h.col[code >> 1];
-        double d = D[code >> 1];
-#pragma unroll 1
-        for (; x < e1; ++x) {
-          const int c0 = col, neg = code << 31;
-          const double v = flip(d, neg);
-          code = x + 1 < e1 ? h.term[x + 1] : 0;
-          col = h.col[code >> 1];
-          d = D[code >> 1];
-          if (c0 != in)
-            Jr[1 + c0] += v;
-          else
-            a += v;
-        }
+        row_sums(h, sig, dq, k, b, tc);
+        row_terms(h, D, k, in, Jr + 1, a);
         A[k] = a;
         B[k] = b;
         Tc[k] = tc;
       }
     }
-    named_sync(t.bar, TEAM_NT);
+    jac_sync<TW>();
     // row coefficients of the dense part, then one pass per column
     const double irho = 1.0 / rho, iS = 1.0 / S, cpm = ct.cpm;
-    for (int k = lane + 32 * wt; k < in; k += TEAM_NT) {
+    for (int k = lane + 32 * wt; k < in; k += NT) {
       A[k] *= rW[in];
       B[k] *= iS;
       wd[k] = m.W[k] * wd[k] * irho * irho;
       bS[k] = wd[k] * (rho / S);
     }
-    named_sync(t.bar, TEAM_NT);
+    jac_sync<TW>();
     const double HwJ = ct.Hw * RU * T, CPwJ = ct.CPw * RU, rcp = rho * cpm * RU;
     const double hfac = RU * T / rcp, g2 = HwJ / (rcp * rcp);
     bool ok = true;
-    for (int c = lane + 32 * wt; c < N; c += TEAM_NT) {
+    for (int c = lane + 32 * wt; c < N; c += NT) {
       double dh = 0.0, drcp, extra = 0.0;
-      LT *Jc = t.J + (size_t)c * ld;
       if (c == 0) {
         const double x = rho * invT;
 #pragma unroll 1
@@ -1155,7 +1168,7 @@ struct TeamMassFrac {
           dh = t_fma(hs[k], v, dh);
           const double w = t_fma(t_mul(m.W[k], irho), v, t_mul(wd[k], x));
           ok &= isfinite(w);
-          Jc[1 + k] = LT(w);
+          put(1 + k, c, w);
         }
         drcp = cpm * RU * (-rho * invT) + rho * ct.dcpm * RU;
         extra = -CPwJ / rcp;
@@ -1168,7 +1181,7 @@ struct TeamMassFrac {
           dh = t_fma(hs[k], v, dh);
           const double w = t_fma(t_mul(m.W[k], irho), v, t_mul(bS[k], mj));
           ok &= isfinite(w);
-          Jc[1 + k] = LT(w);
+          put(1 + k, c, w);
         }
         const double cpin = t_mul(cpk[in], m.invW[in]);
         drcp = t_fma(t_mul(cpm, RU), -rho * mj / S,
@@ -1176,19 +1189,23 @@ struct TeamMassFrac {
       }
       const double w = t_fma(g2, drcp, t_fma(-hfac, dh, extra));
       ok &= isfinite(w);
-      Jc[0] = LT(w);
+      put(0, c, w);
     }
     if (!G::all(ok) && lane == 0) ct.ret[wt] = 4;
   }
 
-  __device__ __forceinline__ static double flip(double x, int sign) {
-    return __hiloint2double(__double2hiint(x) ^ sign, __double2loint(x));
+  template <int TW>
+  __device__ __forceinline__ void jac_sync() const {
+    if constexpr (TW == 1)
+      __syncwarp();
+    else
+      named_sync(t.bar, 32 * TW);
   }
 };
 
 // E1 = gamma/h - J and E2 = (alpha + i beta)/h - J from J's columns, then the
 // factorisations; the results in ctl->ret
-template <typename LT>
+template <typename LT, bool PIVOT>
 __device__ void team_factor(int N, const TeamBuf<LT> &t, int wt) {
   const int lane = threadIdx.x & 31, ld = t.ld;
   const double h = t.ctl->h;
@@ -1215,7 +1232,8 @@ __device__ void team_factor(int N, const TeamBuf<LT> &t, int wt) {
     }
   }
   named_sync(t.bar, TEAM_NT);
-  const int r = wt == 0 ? team_lu_real<LT>(N, ld, t.E1, t.p1) : team_lu_cplx<LT>(N, t, wt);
+  const int r = wt == 0 ? team_lu_real<LT, PIVOT>(N, ld, t.E1, t.p1, t.d1)
+                        : team_lu_cplx<LT, PIVOT>(N, t, wt);
   if (lane == 0) t.ctl->ret[wt] = r;
 }
 
@@ -1228,7 +1246,7 @@ __device__ __forceinline__ void team_exec(int cmd, int wt, const Form &f) {
   } else if (cmd == TEAM_JAC) {
     f.jac(wt);
   } else if (cmd == TEAM_FACTOR) {
-    team_factor<LT>(f.n(), t, wt);
+    team_factor<LT, Form::PIVOT>(f.n(), t, wt);
   } else if (cmd == TEAM_SOLVE && wt == 1) {
     WVecT<2> xr, xi;
     vec_load(f.n(), t.C(1), xr);
@@ -1334,21 +1352,21 @@ struct TeamSys {
     const TeamBuf<LT> &t = f.t;
     if ((threadIdx.x & 31) == 0) t.ctl->h = h;
     post(TEAM_FACTOR);
-    team_factor<LT>(n(), t, 0);
+    team_factor<LT, Form::PIVOT>(n(), t, 0);
     done();
     const int rc = t.ctl->ret[0] ? t.ctl->ret[0] : t.ctl->ret[1];
     __syncwarp();
     return rc;
   }
   __device__ __forceinline__ void solve_real(const WarpBuf<LT> &, WV &x) const {
-    team_solve_real<LT>(n(), f.t.ld, f.t.E1, f.t.p1, x);
+    team_solve_real<LT>(n(), f.t.ld, f.t.E1, f.t.p1, f.t.d1, x);
   }
   __device__ __forceinline__ void solve_both(const WarpBuf<LT> &, WV &x, WV &xr, WV &xi) const {
     const TeamBuf<LT> &t = f.t;
     vec_store(n(), t.C(1), xr);
     vec_store(n(), t.g(1), xi);
     post(TEAM_SOLVE);
-    team_solve_real<LT>(n(), t.ld, t.E1, t.p1, x);
+    team_solve_real<LT>(n(), t.ld, t.E1, t.p1, t.d1, x);
     done();
     vec_load(n(), t.C(1), xr);
     vec_load(n(), t.g(1), xi);

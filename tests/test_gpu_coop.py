@@ -74,15 +74,15 @@ def test_other_mechanism_forms_give_the_per_thread_bits(form, lu_fp32):
 
 
 def test_both_sides_of_the_size_rule_give_the_same_bits():
-    """A batch of 6145 states (per thread) and its first 6144 (per block)."""
+    """A batch of 5633 states (per thread) and its first 5632 (per block)."""
     m = synth.make_mechanism("h2")
     mg = kin.Mechanism(m)
-    st = synth.make_states(m, 6145, 3)
+    st = synth.make_states(m, 5633, 3)
     a = _run(mg, st.Y, st.T, st.P, 1e-7, layout="plain")
-    sub = st.subset(np.arange(6144))
+    sub = st.subset(np.arange(5632))
     b = _run(mg, sub.Y, sub.T, sub.P, 1e-7, layout="plain")
     for x, y in zip(a, b):
-        np.testing.assert_array_equal(x[..., :6144], y)
+        np.testing.assert_array_equal(x[..., :5632], y)
 
 
 def test_failing_states_and_a_bad_order_are_reported_alike():
