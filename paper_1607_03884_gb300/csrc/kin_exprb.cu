@@ -82,16 +82,26 @@ struct XWork {
   int nfast;     // its size in doubles
 };
 
+// A warp's shared memory: the chemistry's buffers of kin_team.cuh for one warp
+// (C, g, q, the Jacobian's scratch) and, for small mechanisms, the assembly
+// matrix, which is in the global slot otherwise.
+constexpr int XSMALL = 16;
+__host__ __device__ inline size_t xwarp_bytes(const MechLayout &L) {
+  size_t d = 2 * (size_t)team_nv(L.ns) + L.nr + team_js_doubles(L);
+  if (L.ns <= XSMALL) d += (size_t)L.ns * team_ld(L.ns);
+  return ((sizeof(TeamCtl) + 15) / 16 * 16 + d * sizeof(double) + 15) / 16 * 16;
+}
+
 __host__ __device__ inline int xS(int N) { return (N + XKP + 2) & ~1; }
 __host__ __device__ inline size_t xslot_doubles(int N) {
-  size_t d = (size_t)warp_slot_mats(sizeof(double)) * N * (N + 1);  // J, E2r, E2i
+  size_t d = 2 * (size_t)N * (N + 1);                               // J, assembly matrix
   d += 2 * (size_t)(N + 1) * N + xmf_doubles(N) + 2 * (size_t)N;    // V, H, mf, half, vd
   return (d + 31) / 32 * 32;
 }
 
 __device__ XWork carve_xwork(double *slot, int N) {
   XWork w;
-  double *p = slot + (size_t)warp_slot_mats(sizeof(double)) * N * (N + 1);
+  double *p = slot + 2 * (size_t)N * (N + 1);
   w.V = p;
   p += (size_t)(N + 1) * N;
   w.H = p;
@@ -141,14 +151,14 @@ __device__ __forceinline__ void xstore(int N, double *p, const XV &x) {
   }
 }
 
-// y = J x, J row-major (ld) and x in global memory
+// y = J x, J by columns (entry (i, c) at c * ld + i: coalesced), x in memory
 __device__ void xmatvec(int N, int ld, const double *J, const double *x, XV &y) {
 #pragma unroll
   for (int r = 0; r < XWR; ++r) {
     const int g = XG::lane() + XL * r;
     double s = 0.0;
     if (g < N)
-      for (int c = 0; c < N; ++c) s += J[g * ld + c] * x[c];
+      for (int c = 0; c < N; ++c) s += J[c * ld + g] * x[c];
     y.v[r] = s;
   }
 }
@@ -250,6 +260,52 @@ __device__ void xproduct(int N, int m, double beta, const XWork &w, const double
   }
 }
 
+// The chemistry of one warp: rates as the teams evaluate them, the Jacobian
+// assembled by the one warp without atomics.
+struct XChem {
+  const MechView &m;
+  const HotTables &h;
+  const TeamBuf<double> &t;
+  __device__ __forceinline__ int rates(double P, const XV &y, XV &f) const {
+    XG::sync();
+    const int rc = team_rhs<>(m, h, t.C(0), t.g(0), t.q(0), P, y, f);
+    XG::sync();
+    return rc;
+  }
+  // also the Jacobian, into t.J
+  __device__ __noinline__ int jacobian(double P, const XV &y, XV &f) const {
+    const TeamMassFrac<double> c{m, h, t};
+    XG::sync();
+    if (XG::lane() == 0) t.ctl->P = P;
+    XG::sync();
+    c.jac_prepare(y);
+    XG::sync();
+    double *J = t.J;
+    const int ld = t.ld;
+    c.jac_out<1>(0, [J, ld](int i, int k, double v) { J[k * ld + i] = v; });
+    XG::sync();
+    vec_load(m.ns, t.g(0), f);
+    const int rc = t.ctl->ret[0];
+    XG::sync();
+    return rc;
+  }
+};
+
+__device__ __forceinline__ TeamBuf<double> xcarve(const MechLayout &L, unsigned char *p,
+                                                  double *slot) {
+  const int N = L.ns;
+  TeamBuf<double> t{};
+  t.ld = team_ld(N);
+  t.nv = team_nv(N);
+  t.wstride = 2 * t.nv + L.nr;
+  t.ctl = reinterpret_cast<TeamCtl *>(p);
+  t.w0 = reinterpret_cast<double *>(p + (sizeof(TeamCtl) + 15) / 16 * 16);
+  t.js = t.w0 + t.wstride;
+  t.J = slot;
+  t.Jd = N <= XSMALL ? t.js + team_js_doubles(L) : slot + (size_t)N * (N + 1);
+  return t;
+}
+
 struct XProducts {
   int np, kmax;
   int k[3];
@@ -346,11 +402,11 @@ __device__ void xremainder(int N, int ld, const double *J, const XV &U, const XV
 
 // one attempt: 0 done (unew, uhat), 1 a stage was not finite, 2 a matrix
 // function failed
-__device__ int xstep(const MechView &m, const WarpBuf<double> &b, double P, const XWork &w,
+__device__ int xstep(const XChem &x, double P, const XWork &w,
                      const XV &y, const XV &fy, double h, const XV &scal, double kappa, XV &unew,
                      XV &uhat, int &nf, int &kdim) {
-  const int N = m.ns, ld = b.ld;
-  const double *J = b.J;
+  const int N = x.m.ns, ld = x.t.ld;
+  const double *J = x.t.J;
   const XProducts PF = {1, 1, {1, 0, 0}, {1.0, 0.0, 0.0}};
   const XProducts PD2 = {3, 4, {1, 3, 4}, {1.0, 16.0, 48.0}};
   const XProducts PD3 = {2, 4, {3, 4, 0}, {2.0, 12.0, 0.0}};
@@ -373,7 +429,7 @@ __device__ int xstep(const MechView &m, const WarpBuf<double> &b, double P, cons
 #pragma unroll
   for (int r = 0; r < XWR; ++r) U.v[r] = y.v[r] + 0.5 * h * half.v[r];
   nf++;
-  if (warp_chem<XL, double>(m, b, P, U, F, false)) return 1;
+  if (x.rates(P, U, F)) return 1;
   xremainder(N, ld, J, U, y, F, fy, w, D);
   mk = xarnoldi(N, ld, J, D, h, PD2, scal, kappa, w, beta, Z);
   if (mk < 0) return 2;
@@ -391,7 +447,7 @@ __device__ int xstep(const MechView &m, const WarpBuf<double> &b, double P, cons
 #pragma unroll
   for (int r = 0; r < XWR; ++r) U.v[r] = y.v[r] + h * full.v[r] + h * q1.v[r];
   nf++;
-  if (warp_chem<XL, double>(m, b, P, U, F, false)) return 1;
+  if (x.rates(P, U, F)) return 1;
   xremainder(N, ld, J, U, y, F, fy, w, D);
   mk = xarnoldi(N, ld, J, D, h, PD3, scal, kappa, w, beta, Z);
   if (mk < 0) return 2;
@@ -420,14 +476,14 @@ struct XCount {
 
 // One state from y (in: [T, Y_0 .. Y_{ns-2}], out: the state at dt or at
 // its last accepted point).
-__device__ XCount xintegrate(const MechView &m, const WarpBuf<double> &b, double P,
-                             const XWork &w, const XParams &p, int64_t idx, XV &y) {
-  const int N = m.ns;
+__device__ XCount xintegrate(const XChem &ch, double P, const XWork &w,
+                             const XParams &p, int64_t idx, XV &y) {
+  const int N = ch.m.ns;
   XCount c = {0, 0, 0, 0, 0, 0, 0, 0};
   XV fy, scal, unew, uhat;
   c.nfcn = 1;
   c.njac = 1;
-  if (warp_chem<XL, double>(m, b, P, y, fy, true)) {
+  if (ch.jacobian(P, y, fy)) {
     c.status = 4;
     return c;
   }
@@ -443,7 +499,7 @@ __device__ XCount xintegrate(const MechView &m, const WarpBuf<double> &b, double
     XV u, fu;
 #pragma unroll
     for (int r = 0; r < XWR; ++r) u.v[r] = y.v[r] + h0 * fy.v[r];
-    const int rc = warp_chem<XL, double>(m, b, P, u, fu, false);
+    const int rc = ch.rates(P, u, fu);
     c.nfcn++;
     if (rc) {
       h = 0.01 * h0;
@@ -477,7 +533,7 @@ __device__ XCount xintegrate(const MechView &m, const WarpBuf<double> &b, double
 #pragma unroll
     for (int r = 0; r < XWR; ++r) scal.v[r] = p.atol + p.rtol * fabs(y.v[r]);
     int nf = 0, kd = 0;
-    const int rc = xstep(m, b, P, w, y, fy, h, scal, p.kappa, unew, uhat, nf, kd);
+    const int rc = xstep(ch, P, w, y, fy, h, scal, p.kappa, unew, uhat, nf, kd);
     c.nfcn += nf;
     c.narn += 3;
     c.kdim += kd;
@@ -506,7 +562,7 @@ __device__ XCount xintegrate(const MechView &m, const WarpBuf<double> &b, double
       if (last) return c;
       c.nfcn++;
       c.njac++;
-      if (warp_chem<XL, double>(m, b, P, y, fy, true)) {
+      if (ch.jacobian(P, y, fy)) {
         c.status = 4;
         return c;
       }
@@ -532,28 +588,32 @@ struct XArgs {
   XParams p;
   double *scratch;
   int64_t slots;
+  const unsigned char *hot;  // the tables of kin_team.cuh
+  int hot_smem;              // copied to shared memory by each block
 };
 
 __global__ void __launch_bounds__(256) k_integrate_exprb(XArgs a) {
-  extern __shared__ double smem[];
+  extern __shared__ __align__(16) unsigned char xsmem[];
   const MechView m = make_view(a.L, a.tab, a.itab);
   const int N = m.ns, lane = XG::lane(), grp = (int)(threadIdx.x / XL);
   const int64_t n = a.p.n;
-  char *base = reinterpret_cast<char *>(smem) + (size_t)grp * warp_buf_bytes(N, m.nr, sizeof(double));
+  const HotTables h = stage_hot(a.L, a.hot, a.hot_smem != 0, xsmem);
+  const size_t hb = a.hot_smem ? hot_offsets(a.L).bytes : 0;
   const int64_t slot = (int64_t)blockIdx.x * (blockDim.x / XL) + grp;  // < slots (launch)
   double *gs = a.scratch + slot * (int64_t)xslot_doubles(N);
-  const WarpBuf<double> b = carve_warp_buf<double>(base, N, m.nr, gs);
+  const TeamBuf<double> t = xcarve(a.L, xsmem + hb + grp * xwarp_bytes(a.L), gs);
+  const XChem ch{m, h, t};
   XWork w = carve_xwork(gs, N);
-  // E1's shared memory is free outside the Jacobian's assembly
-  w.fast = b.E1;
-  w.nfast = (int)(warp_e1_bytes(N, sizeof(double)) / sizeof(double));
+  // the Jacobian's scratch is free outside its assembly
+  w.fast = t.js;
+  w.nfast = (int)team_js_doubles(a.L);
   unsigned long long *queue = a.totals + 9;
   for (;;) {
-    unsigned long long t = 0;
-    if (lane == 0) t = atomicAdd(queue, 1ull);
-    t = XG::bcast(t, 0);
-    if (t >= (unsigned long long)n) break;
-    const int64_t idx = (int64_t)t;
+    unsigned long long q = 0;
+    if (lane == 0) q = atomicAdd(queue, 1ull);
+    q = XG::bcast(q, 0);
+    if (q >= (unsigned long long)n) break;
+    const int64_t idx = (int64_t)q;
     const double P = a.P[idx];
     XV y;
 #pragma unroll
@@ -561,7 +621,7 @@ __global__ void __launch_bounds__(256) k_integrate_exprb(XArgs a) {
       const int g = lane + XL * r;
       y.v[r] = (g == 0) ? a.T[idx] : (g < N ? a.Y[(int64_t)(g - 1) * n + idx] : 0.0);
     }
-    const XCount c = xintegrate(m, b, P, w, a.p, idx, y);
+    const XCount c = xintegrate(ch, P, w, a.p, idx, y);
     double sum = 0.0;
 #pragma unroll
     for (int r = 0; r < XWR; ++r) {
@@ -606,33 +666,36 @@ __global__ void k_exprb_phi(const double *H, int m, int p, double tau, double *o
 
 // unit entry: the right-hand side (with and without the Jacobian's assembly)
 // and the analytical Jacobian the method uses, one state per warp
-__global__ void k_exprb_chem(MechLayout L, const double *tab, const int *itab, const double *y,
+__global__ void k_exprb_chem(MechLayout L, const double *tab, const int *itab,
+                             const unsigned char *hot, int hot_smem, const double *y,
                              const double *P, int64_t n, double *f, double *f2, double *J,
                              double *scratch, int64_t slots) {
-  extern __shared__ double smem[];
+  extern __shared__ __align__(16) unsigned char xsmem[];
   const MechView m = make_view(L, tab, itab);
-  const int N = m.ns, lane = XG::lane(), grp = (int)(threadIdx.x / XL);
-  const int64_t slot = (int64_t)blockIdx.x * (blockDim.x / XL) + grp;
+  const int N = m.ns, lane = XG::lane();
+  const HotTables h = stage_hot(L, hot, hot_smem != 0, xsmem);
+  const int64_t slot = (int64_t)blockIdx.x;
   if (slot >= slots) return;
-  char *base = reinterpret_cast<char *>(smem) + (size_t)grp * warp_buf_bytes(N, m.nr, sizeof(double));
   double *gs = scratch + slot * (int64_t)xslot_doubles(N);
-  const WarpBuf<double> b = carve_warp_buf<double>(base, N, m.nr, gs);
-  for (int64_t i = slot; i < n; i += (int64_t)gridDim.x * (blockDim.x / XL)) {
+  const TeamBuf<double> t = xcarve(L, xsmem + (hot_smem ? hot_offsets(L).bytes : 0), gs);
+  const XChem ch{m, h, t};
+  for (int64_t i = slot; i < n; i += (int64_t)gridDim.x) {
     XV yy, ff;
 #pragma unroll
     for (int r = 0; r < XWR; ++r) {
       const int g = lane + XL * r;
       yy.v[r] = g < N ? y[(int64_t)g * n + i] : 0.0;
+      ff.v[r] = 0.0;
     }
-    warp_chem<XL, double>(m, b, P[i], yy, ff, true);
+    ch.jacobian(P[i], yy, ff);
 #pragma unroll
     for (int r = 0; r < XWR; ++r) {
       const int g = lane + XL * r;
       if (g < N) f[(int64_t)g * n + i] = ff.v[r];
     }
-    for (int e = lane; e < N * N; e += XL) J[(int64_t)e * n + i] = b.J[(e / N) * b.ld + e % N];
+    for (int e = lane; e < N * N; e += XL) J[(int64_t)e * n + i] = t.J[(e % N) * t.ld + e / N];
     XG::sync();
-    warp_chem<XL, double>(m, b, P[i], yy, ff, false);
+    ch.rates(P[i], yy, ff);
 #pragma unroll
     for (int r = 0; r < XWR; ++r) {
       const int g = lane + XL * r;
@@ -640,6 +703,16 @@ __global__ void k_exprb_chem(MechLayout L, const double *tab, const int *itab, c
     }
     XG::sync();
   }
+}
+
+// whether the tables are staged, and their bytes; false when not even one
+// warp's buffers fit
+bool xshape(const MechLayout &L, int &hot_smem, size_t &fixed) {
+  const size_t budget = 227 * 1024, hot = hot_offsets(L).bytes, per = xwarp_bytes(L);
+  if (per > budget) return false;
+  hot_smem = hot + per <= budget;
+  fixed = hot_smem ? hot : 0;
+  return true;
 }
 
 }  // namespace
@@ -651,6 +724,7 @@ struct kin_exprb {
   int *d_itab = nullptr;
   unsigned long long *d_totals = nullptr;
   double *d_scratch = nullptr;
+  unsigned char *d_hot = nullptr;
   int64_t slots = 0;
   cudaStream_t last_stream = nullptr;
 };
@@ -661,6 +735,7 @@ extern "C" void kin_exprb_destroy(kin_exprb *x) {
   cudaFree(x->d_itab);
   cudaFree(x->d_totals);
   cudaFree(x->d_scratch);
+  cudaFree(x->d_hot);
   delete x;
 }
 
@@ -676,6 +751,7 @@ extern "C" int kin_exprb_create(const kin_mech_desc *desc, kin_exprb **out) {
   int dev = 0, sms = 0;
   KIN_CUDA_TRY(cudaGetDevice(&dev));
   KIN_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  const std::vector<unsigned char> hot = build_hot(L, dt, it);
   kin_exprb *x = new kin_exprb();
   x->device = dev;
   x->L = L;
@@ -684,12 +760,14 @@ extern "C" int kin_exprb_create(const kin_mech_desc *desc, kin_exprb **out) {
   if (cudaMalloc(&x->d_tab, sizeof(double) * L.nd) != cudaSuccess ||
       cudaMalloc(&x->d_itab, sizeof(int) * L.ni) != cudaSuccess ||
       cudaMalloc(&x->d_totals, sizeof(unsigned long long) * 16) != cudaSuccess ||
+      cudaMalloc(&x->d_hot, hot.size()) != cudaSuccess ||
       cudaMalloc(&x->d_scratch, sbytes) != cudaSuccess) {
     (void)cudaGetLastError();
     kin_exprb_destroy(x);
     return KIN_ERR_NOMEM;
   }
-  if (cudaMemcpy(x->d_tab, dt.data(), sizeof(double) * L.nd, cudaMemcpyHostToDevice) !=
+  if (cudaMemcpy(x->d_hot, hot.data(), hot.size(), cudaMemcpyHostToDevice) != cudaSuccess ||
+      cudaMemcpy(x->d_tab, dt.data(), sizeof(double) * L.nd, cudaMemcpyHostToDevice) !=
           cudaSuccess ||
       cudaMemcpy(x->d_itab, it.data(), sizeof(int) * L.ni, cudaMemcpyHostToDevice) !=
           cudaSuccess ||
@@ -738,11 +816,14 @@ extern "C" int kin_integrate_exprb(kin_exprb *x, double *Y, double *T, const dou
   a.p.h0 = h0;
   a.scratch = x->d_scratch;
   a.slots = x->slots;
-  const size_t budget = 227 * 1024, per = warp_buf_bytes(x->L.ns, x->L.nr, sizeof(double));
+  a.hot = x->d_hot;
+  size_t fixed = 0;
+  if (!xshape(x->L, a.hot_smem, fixed)) return KIN_ERR_UNSUPPORTED;
+  const size_t budget = 227 * 1024, per = xwarp_bytes(x->L);
   auto kern = k_integrate_exprb;
   int warps = 0, per_sm = 0;
   for (int wp = 8; wp >= 1; wp >>= 1) {
-    const size_t smw = (size_t)wp * per;
+    const size_t smw = fixed + (size_t)wp * per;
     if (smw > budget) continue;
     KIN_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smw));
     int nb = 0;
@@ -753,7 +834,7 @@ extern "C" int kin_integrate_exprb(kin_exprb *x, double *Y, double *T, const dou
     }
   }
   if (warps < 1 || per_sm < 1) return KIN_ERR_UNSUPPORTED;
-  const size_t sm = (size_t)warps * per;
+  const size_t sm = fixed + (size_t)warps * per;
   KIN_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
   int64_t grid = (int64_t)sms * per_sm;
   const int64_t need = (n + warps - 1) / warps;
@@ -787,12 +868,16 @@ extern "C" int kin_exprb_chem(kin_exprb *x, const double *y, const double *P, in
                               double *f, double *f_rates, double *J, void *stream) {
   if (!x || n < 0 || (n > 0 && (!y || !P || !f || !f_rates || !J))) return KIN_ERR_INVALID_ARG;
   if (n == 0) return KIN_OK;
-  const size_t sm = warp_buf_bytes(x->L.ns, x->L.nr, sizeof(double));
+  int hot_smem = 0;
+  size_t fixed = 0;
+  if (!xshape(x->L, hot_smem, fixed)) return KIN_ERR_UNSUPPORTED;
+  const size_t sm = fixed + xwarp_bytes(x->L);
   KIN_CUDA_TRY(cudaFuncSetAttribute(k_exprb_chem, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     (int)sm));
   const int64_t grid = n < x->slots ? n : x->slots;
   k_exprb_chem<<<(unsigned)grid, XL, sm, (cudaStream_t)stream>>>(
-      x->L, x->d_tab, x->d_itab, y, P, n, f, f_rates, J, x->d_scratch, x->slots);
+      x->L, x->d_tab, x->d_itab, x->d_hot, hot_smem, y, P, n, f, f_rates, J, x->d_scratch,
+      x->slots);
   KIN_CUDA_TRY(cudaGetLastError());
   return KIN_OK;
 }

@@ -1015,45 +1015,14 @@ struct kin_mlp {
   float *xg = nullptr, *tg = nullptr;  // gathered minibatch rows (train_step_rows)
   int *err = nullptr;                  // set by a tensor-core GEMM whose wait expired
   __nv_bfloat16 *xb = nullptr, *hb[LAYERS] = {}, *gb = nullptr, *gb2 = nullptr;
+  // Tensor maps of the fused path's operands, built with the buffers they
+  // describe: encoding two per GEMM took as long as launching it.  Activations
+  // and gradients span the buffers' capacity; rows past a batch give
+  // accumulator rows that are never stored.
+  CUtensorMap mx, mh[LAYERS], mg[2][2];  // mg: buffer gb / gb2, width doutp / width
+  CUtensorMap mw[LAYERS], mwt[LAYERS];   // weight blocks [K][N] and transposed [N][K]
+  bool maps = false;
 };
-
-static int mlp_reserve(kin_mlp *n, int64_t rows) {
-  if (rows <= n->cap) return KIN_OK;
-  cudaFree(n->xg);
-  cudaFree(n->tg);
-  n->xg = n->tg = nullptr;
-  cudaFree(n->xf);
-  cudaFree(n->xb);
-  cudaFree(n->C);
-  cudaFree(n->g);
-  cudaFree(n->dH);
-  cudaFree(n->gb);
-  cudaFree(n->gb2);
-  for (int l = 0; l < LAYERS; ++l) {
-    cudaFree(n->a[l]);
-    cudaFree(n->hf[l]);
-    cudaFree(n->hb[l]);
-  }
-  n->cap = 0;
-  const int64_t wmax = n->width > n->doutp ? n->width : n->doutp;
-  KIN_CUDA_TRY(cudaMalloc(&n->xg, sizeof(float) * rows * n->din));
-  KIN_CUDA_TRY(cudaMalloc(&n->tg, sizeof(float) * rows * n->dout));
-  KIN_CUDA_TRY(cudaMalloc(&n->xf, sizeof(float) * rows * n->dinp));
-  KIN_CUDA_TRY(cudaMalloc(&n->xb, sizeof(__nv_bfloat16) * rows * n->dinp));
-  KIN_CUDA_TRY(cudaMalloc(&n->C, sizeof(float) * rows * wmax));
-  KIN_CUDA_TRY(cudaMalloc(&n->g, sizeof(float) * rows * wmax));
-  KIN_CUDA_TRY(cudaMalloc(&n->dH, sizeof(float) * rows * wmax));
-  KIN_CUDA_TRY(cudaMalloc(&n->gb, sizeof(__nv_bfloat16) * rows * wmax));
-  KIN_CUDA_TRY(cudaMalloc(&n->gb2, sizeof(__nv_bfloat16) * rows * wmax));
-  for (int l = 0; l < LAYERS; ++l) {
-    KIN_CUDA_TRY(cudaMalloc(&n->a[l], sizeof(float) * rows * n->N[l]));
-    KIN_CUDA_TRY(cudaMalloc(&n->hf[l], sizeof(float) * rows * n->N[l]));
-    KIN_CUDA_TRY(cudaMalloc(&n->hb[l], sizeof(__nv_bfloat16) * rows * n->N[l]));
-  }
-  n->y = n->hf[LAYERS - 1];
-  n->cap = rows;
-  return KIN_OK;
-}
 
 // cuTensorMapEncodeTiled through the runtime's driver entry point (no link
 // against the driver library); null when unavailable
@@ -1092,6 +1061,61 @@ static bool make_tmap(CUtensorMap *m, const void *base, int64_t rows, int64_t co
          CUDA_SUCCESS;
 }
 
+static bool mlp_maps(kin_mlp *n) {
+  if (n->precision != 0 || n->width % 8 != 0) return false;
+  bool ok = make_tmap(&n->mx, n->xb, n->cap, n->dinp, n->dinp, true);
+  for (int l = 0; l < LAYERS; ++l) {
+    ok = ok && make_tmap(&n->mh[l], n->hb[l], n->cap, n->N[l], n->N[l], true);
+    ok = ok && make_tmap(&n->mw[l], n->wb + n->woff[l], n->K[l], n->N[l], n->N[l], true);
+    ok = ok && make_tmap(&n->mwt[l], n->wbt + n->woff[l], n->N[l], n->K[l], n->K[l], true);
+  }
+  for (int q = 0; q < 2; ++q)
+    for (int w = 0; w < 2; ++w) {
+      const int ld = w ? n->width : n->doutp;
+      ok = ok && make_tmap(&n->mg[q][w], q ? n->gb2 : n->gb, n->cap, ld, ld, true);
+    }
+  return ok;
+}
+
+static int mlp_reserve(kin_mlp *n, int64_t rows) {
+  if (rows <= n->cap) return KIN_OK;
+  cudaFree(n->xg);
+  cudaFree(n->tg);
+  n->xg = n->tg = nullptr;
+  cudaFree(n->xf);
+  cudaFree(n->xb);
+  cudaFree(n->C);
+  cudaFree(n->g);
+  cudaFree(n->dH);
+  cudaFree(n->gb);
+  cudaFree(n->gb2);
+  for (int l = 0; l < LAYERS; ++l) {
+    cudaFree(n->a[l]);
+    cudaFree(n->hf[l]);
+    cudaFree(n->hb[l]);
+  }
+  n->cap = 0;
+  const int64_t wmax = n->width > n->doutp ? n->width : n->doutp;
+  KIN_CUDA_TRY(cudaMalloc(&n->xg, sizeof(float) * rows * n->din));
+  KIN_CUDA_TRY(cudaMalloc(&n->tg, sizeof(float) * rows * n->dout));
+  KIN_CUDA_TRY(cudaMalloc(&n->xf, sizeof(float) * rows * n->dinp));
+  KIN_CUDA_TRY(cudaMalloc(&n->xb, sizeof(__nv_bfloat16) * rows * n->dinp));
+  KIN_CUDA_TRY(cudaMalloc(&n->C, sizeof(float) * rows * wmax));
+  KIN_CUDA_TRY(cudaMalloc(&n->g, sizeof(float) * rows * wmax));
+  KIN_CUDA_TRY(cudaMalloc(&n->dH, sizeof(float) * rows * wmax));
+  KIN_CUDA_TRY(cudaMalloc(&n->gb, sizeof(__nv_bfloat16) * rows * wmax));
+  KIN_CUDA_TRY(cudaMalloc(&n->gb2, sizeof(__nv_bfloat16) * rows * wmax));
+  for (int l = 0; l < LAYERS; ++l) {
+    KIN_CUDA_TRY(cudaMalloc(&n->a[l], sizeof(float) * rows * n->N[l]));
+    KIN_CUDA_TRY(cudaMalloc(&n->hf[l], sizeof(float) * rows * n->N[l]));
+    KIN_CUDA_TRY(cudaMalloc(&n->hb[l], sizeof(__nv_bfloat16) * rows * n->N[l]));
+  }
+  n->y = n->hf[LAYERS - 1];
+  n->cap = rows;
+  n->maps = mlp_maps(n);
+  return KIN_OK;
+}
+
 // TMA operand loads (1) or the threads' copies only (0): a build-time knob
 #ifndef KIN_MLP_TMA
 #define KIN_MLP_TMA 1
@@ -1113,7 +1137,7 @@ static void gemm(const kin_mlp *n, cudaStream_t st, int M, int N, int K, bool bf
     const int64_t tiles = (int64_t)grid.x * grid.y, kt = (K + TC_BK - 1) / TC_BK;
     int S = 1;
     if (tiles < 2 * 152 && kt >= 8) {
-      S = (int)std::min<int64_t>(kt / 4, (2 * 152 + tiles - 1) / tiles);
+      S = (int)std::min<int64_t>(kt / 2, (2 * 152 + tiles - 1) / tiles);
       while (S > 1 && (int64_t)S * M * N > n->ws_floats) --S;
     }
     if (S > 1) {
@@ -1144,11 +1168,10 @@ static bool mlp_fused(const kin_mlp *n) {
 }
 
 static int gemm_kk(const kin_mlp *n, cudaStream_t st, int64_t M, int N, int K,
-                   const __nv_bfloat16 *A, const __nv_bfloat16 *B, const Epilogue &ep) {
-  CUtensorMap tmA, tmB;
-  if (!make_tmap(&tmA, A, M, K, K, true) || !make_tmap(&tmB, B, N, K, K, true)) return KIN_ERR_CUDA;
+                   const CUtensorMap &A, const CUtensorMap &B, const Epilogue &ep) {
+  if (!n->maps) return KIN_ERR_CUDA;
   const dim3 grid((unsigned)((M + TC_BM - 1) / TC_BM), (unsigned)((N + TC_BN - 1) / TC_BN), 1);
-  k_gemm_kk<<<grid, KK_THREADS, KK_SMEM, st>>>(M, N, K, n->err, tmA, tmB, ep);
+  k_gemm_kk<<<grid, KK_THREADS, KK_SMEM, st>>>(M, N, K, n->err, A, B, ep);
   KIN_CUDA_TRY(cudaGetLastError());
   return KIN_OK;
 }
@@ -1166,8 +1189,7 @@ static int mlp_forward_fused(kin_mlp *n, int64_t M, cudaStream_t st, bool keep, 
     }
     ep.bias = n->p + n->boff[l];
     ep.dout = n->dout;
-    const int rc = gemm_kk(n, st, M, n->N[l], n->K[l], l ? n->hb[l - 1] : n->xb,
-                           n->wbt + n->woff[l], ep);
+    const int rc = gemm_kk(n, st, M, n->N[l], n->K[l], l ? n->mh[l - 1] : n->mx, n->mwt[l], ep);
     if (rc) return rc;
   }
   return KIN_OK;
@@ -1191,6 +1213,7 @@ static int mlp_grad_fused(kin_mlp *n, int64_t M, const float *T, const int32_t *
   // gradient is written while its own gradient is read
   float *g = n->g, *g2 = n->dH;
   __nv_bfloat16 *gb = n->gb, *gb2 = n->gb2;
+  int cur = 0;  // the buffer pair holding layer l's gradient
   for (int l = LAYERS - 1; l >= 0; --l) {
     const int K = n->K[l], N = n->N[l];
     gemm(n, st, K, N, (int)M, true, l ? n->hb[l - 1] : n->xb, 1, K, gb, N, 1,
@@ -1202,7 +1225,8 @@ static int mlp_grad_fused(kin_mlp *n, int64_t M, const float *T, const int32_t *
     e.a = n->a[l - 1];
     e.g = g2;
     e.gb = gb2;
-    if ((rc = gemm_kk(n, st, M, K, N, gb, n->wb + n->woff[l], e))) return rc;
+    if ((rc = gemm_kk(n, st, M, K, N, n->mg[cur][l < LAYERS - 1], n->mw[l], e))) return rc;
+    cur ^= 1;
     std::swap(g, g2);
     std::swap(gb, gb2);
   }
