@@ -332,12 +332,23 @@ __global__ void __launch_bounds__(TC_THREADS) k_gemm_tc(int M, int N, int K,
       asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
       if (row < M) {
         float *dst = C + (int64_t)row * ldc + n0 + c0;
+        // whole 16-byte pieces when the rows allow it: a lane's scalar stores
+        // touch one sector each
+        if (!accumulate && n0 + c0 + 16 <= N && ldc % 4 == 0 &&
+            (reinterpret_cast<uintptr_t>(C) & 15) == 0) {
 #pragma unroll
-        for (int j = 0; j < 16; ++j)
-          if (n0 + c0 + j < N) {
-            const float x = __uint_as_float(v[j]);
-            dst[j] = accumulate ? dst[j] + x : x;
-          }
+          for (int q = 0; q < 4; ++q)
+            *reinterpret_cast<float4 *>(dst + 4 * q) =
+                make_float4(__uint_as_float(v[4 * q]), __uint_as_float(v[4 * q + 1]),
+                            __uint_as_float(v[4 * q + 2]), __uint_as_float(v[4 * q + 3]));
+        } else {
+#pragma unroll
+          for (int j = 0; j < 16; ++j)
+            if (n0 + c0 + j < N) {
+              const float x = __uint_as_float(v[j]);
+              dst[j] = accumulate ? dst[j] + x : x;
+            }
+        }
       }
     }
   } else {
@@ -433,12 +444,52 @@ __device__ __forceinline__ void kk_epilogue(const Epilogue &ep, int64_t M, int N
         *reinterpret_cast<uint4 *>(h + o + 8 * q) = *reinterpret_cast<const uint4 *>(b + 8 * q);
     return;
   }
-  int64_t tr = r;
-  if (ep.mode == EP_MSE && ep.rows) {
-    const int32_t s = ep.rows[r];
-    tr = (s >= 0 && (int64_t)s < ep.nrows) ? (int64_t)s : -1;
+  if (ep.mode == EP_MSE) {
+    int64_t tr = r;
+    if (ep.rows) {
+      const int32_t s = ep.rows[r];
+      tr = (s >= 0 && (int64_t)s < ep.nrows) ? (int64_t)s : -1;
+    }
+    const float scale = (float)(M * ep.dout);
+    const float *t = ep.tgt + tr * ep.dout + c0;
+    __align__(16) float g[16];
+    __align__(16) __nv_bfloat16 b[16];
+    float tv[16];
+    // a row's targets 16 bytes at a time when its length allows
+    const bool vec = tr >= 0 && ep.dout % 4 == 0 && c0 + 16 <= ep.dout &&
+                     (reinterpret_cast<uintptr_t>(ep.tgt) & 15) == 0;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      float4 x = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+      if (vec) x = *reinterpret_cast<const float4 *>(t + 4 * q);
+      tv[4 * q] = x.x;
+      tv[4 * q + 1] = x.y;
+      tv[4 * q + 2] = x.z;
+      tv[4 * q + 3] = x.w;
+    }
+    float sq = 0.0f;
+#pragma unroll
+    for (int j = 0; j < 16; ++j) {
+      g[j] = 0.0f;
+      if (j < n && c0 + j < ep.dout) {
+        const float y = __uint_as_float(v[j]) + ep.bias[c0 + j];
+        const float d = y - (vec ? tv[j] : tr >= 0 ? t[j] : 0.0f);
+        g[j] = 2.0f * d / scale;
+        sq += d * d;
+      }
+      b[j] = __float2bfloat16(g[j]);
+    }
+    loss += sq / scale;
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      if (4 * q < n)
+        *reinterpret_cast<float4 *>(ep.g + o + 4 * q) = *reinterpret_cast<const float4 *>(g + 4 * q);
+#pragma unroll
+    for (int q = 0; q < 2; ++q)
+      if (8 * q < n)
+        *reinterpret_cast<uint4 *>(ep.gb + o + 8 * q) = *reinterpret_cast<const uint4 *>(b + 8 * q);
+    return;
   }
-  const float scale = (float)(M * ep.dout);
 #pragma unroll
   for (int j = 0; j < 16; ++j) {
     const int c = c0 + j;
@@ -446,15 +497,6 @@ __device__ __forceinline__ void kk_epilogue(const Epilogue &ep, int64_t M, int N
     const float y = __uint_as_float(v[j]) + ep.bias[c];
     if (ep.mode == EP_OUT) {
       if (c < ep.dout) ep.out[r * ep.dout + c] = y;
-    } else if (ep.mode == EP_MSE) {
-      float g = 0.0f;
-      if (c < ep.dout) {
-        const float d = y - (tr >= 0 ? ep.tgt[tr * ep.dout + c] : 0.0f);
-        g = 2.0f * d / scale;
-        loss += d * d / scale;
-      }
-      ep.g[o + j] = g;
-      ep.gb[o + j] = __float2bfloat16(g);
     } else if (c < ep.dout) {
       const double sd = widen(ep.stdv[c]), mu = widen(ep.mean[c]);
       if (c == 0) {
