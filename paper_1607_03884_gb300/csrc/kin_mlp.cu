@@ -741,7 +741,7 @@ __global__ void __cluster_dims__(CS_CTAS, 1, 1) __launch_bounds__(CS_THREADS)
   const int64_t step = (int64_t)CS_CTAS * (CS_THREADS / 32);
   float s = 0.0f;
   if (c < N) {
-#pragma unroll 4
+#pragma unroll 16
     for (int64_t r = (int64_t)cl.block_rank() * (CS_THREADS / 32) + y; r < M; r += step)
       s += g[r * N + c];
   }
@@ -834,6 +834,7 @@ __global__ void k_splitk_reduce(int M, int N, int S, const float *ws, float *C, 
   if (i >= (int64_t)M * N) return;
   const int m = (int)(i / N), n = (int)(i % N);
   float v = 0.0f;
+#pragma unroll 16
   for (int q = 0; q < S; ++q) v += ws[(int64_t)q * M * N + i];
   float *dst = C + (int64_t)m * ldc + n;
   *dst = accumulate ? *dst + v : v;
