@@ -1,5 +1,5 @@
 // Concentration-based reactor with a sparse LU (kin_conc_* of the C ABI):
-// the host's symbolic analysis, the state-per-group kernel and its launch.
+// the host's symbolic analysis, the state-per-team kernel and its launch.
 // The reformulation is the one the paper proposes for large models (Sec. 3.3,
 // Sec. 4); kin_conc.cuh has the device side and the equations.
 #include <cuda_runtime.h>

@@ -39,7 +39,9 @@
 // 1150 of them per evaluation and eleven evaluations a step; the blocks take
 // 300, and the estimate's evaluation at the accepted dimension also gives the
 // step's products (phi_1 at h/2 is the state before the last doubling), so
-// seven evaluations remain.
+// seven evaluations remain.  The rates and the Jacobian are a team's
+// (kin_team.cuh) with one warp, their tables in shared memory.  Measured (H2
+// states, FP64): 309 -> 147 ms by the blocks, 113 ms with the tables.
 #include <cuda_runtime.h>
 
 #include <cmath>

@@ -444,7 +444,12 @@ struct TeamLaunch {
 };
 
 // teams per block and blocks for a batch; the tables go to shared memory when
-// a team fits beside them.  false when not even one team fits.
+// a team fits beside them.  A team always fits: a mechanism's tables are at
+// most 200 KB (build_tables); a reaction takes 64 bytes there and 12 more per
+// species that it changes and per collision efficiency, and of a team's buffers
+// 24 bytes and 8 per slot and efficiency, beside at most 45 KB of matrices and
+// species vectors.  (Only some 2900 reactions of six slots that change no
+// species at all would not; they are refused.)
 inline bool team_shape(KernelArgs &a, int N, size_t lt, int sms, TeamLaunch &g) {
   const size_t budget = 227 * 1024, tb = team_bytes(a.L, N, lt), hot = hot_offsets(a.L).bytes;
   if (!a.hot || tb > budget) return false;

@@ -23,6 +23,10 @@
 //     and serve all its teams.
 // Every matrix entry sees the same operations in the same order as in a
 // column-by-column elimination, so FP32 matrices factorise to the same bits.
+// Measured on CH4-like states (warp per state -> team): 4000 states, dt =
+// 1e-4 s, FP32 matrices 579 -> 333 ms, the same bits; dt = 1e-6 s, FP64
+// matrices 380 -> 208 ms.  Also tried, FP32: two rows per lane in the trailing
+// update, as FP64 has it, 333 -> 340 ms.
 #pragma once
 #include "kin_warp.cuh"
 

@@ -1,5 +1,8 @@
-// Radau IIA with one state per group of L lanes (L = 4, 8, 16 or 32; the
-// WARP layout), the per-block strategy the paper points to for large models.
+// Radau IIA with one state per group of L lanes (the WARP layout), the
+// per-block strategy the paper points to for large models.  Groups of 4, 8 and
+// 16 lanes use everything here; with 32 lanes the step driver, the vector
+// operations and the rate expressions serve the teams of warps of
+// kin_team.cuh, which bring their own chemistry and linear algebra.
 //
 // The paper's per-thread organisation stores each state's Jacobian and
 // factorisations privately; for large models those overwhelm on-chip memory
@@ -27,12 +30,6 @@
 #include "kin_radau.cuh"
 
 namespace kin {
-
-// Elementary reactions of the rate-only path two per lane per round (1) or
-// one (0): a build-time tuning knob.
-#ifndef KIN_WARP_PAIRED_RATES
-#define KIN_WARP_PAIRED_RATES 0
-#endif
 
 template <int L>
 struct Grp {
@@ -121,12 +118,13 @@ __host__ __device__ inline size_t warp_e1_bytes(int N, size_t lt) {
 
 // Where the complex iteration matrix lives: in the group's shared-memory
 // slice, or after J in the group's global slot, which leaves shared memory
-// to more resident warps while its rows stream through L1/L2.  Measured on
-// 16384 CH4-like states (dt = 1e-4 s): with FP64 matrices the global
-// placement raises the resident warps from 3 to 7 per SM and the rate by
-// 26 %; with FP32 matrices (5 warps per SM in shared memory) it costs 26 %.
-// So FP64 matrices go to the global slot and FP32 ones stay in shared
-// memory (KIN_WARP_E2_GLOBAL_F64 = 0 keeps both in shared memory).
+// to more resident states while its rows stream through L1/L2.  Measured with
+// one warp per state on 16384 CH4-like states (dt = 1e-4 s): with FP64
+// matrices the global placement raised the resident states from 3 to 7 per SM
+// and the rate by 26 %; with FP32 matrices (5 per SM in shared memory) it cost
+// 26 %.  So FP64 matrices go to the global slot and FP32 ones stay in shared
+// memory, for groups and for teams (KIN_WARP_E2_GLOBAL_F64 = 0 keeps both in
+// shared memory).
 #ifndef KIN_WARP_E2_GLOBAL_F64
 #define KIN_WARP_E2_GLOBAL_F64 1
 #endif
@@ -318,8 +316,7 @@ __device__ __noinline__ int warp_chem(const MechView &m, const WarpBuf<LT> &b, d
   // Rates only (most evaluations: Newton stages, error refinement): the
   // falloff reactions, which the device order puts first, in their own
   // rounds (Troe, then third-body), so their branches never split a round of
-  // elementary reactions; then the elementary reactions two per lane per
-  // round, for two independent FP64 chains per lane.
+  // elementary reactions; then the elementary reactions.
   if (!wantJ) {
     for (int i0 = 0; i0 < m.ntroe; i0 += L)
       if (i0 + lane < m.ntroe)
@@ -327,19 +324,8 @@ __device__ __noinline__ int warp_chem(const MechView &m, const WarpBuf<LT> &b, d
     for (int i0 = m.ntroe; i0 < m.nfall; i0 += L)
       if (i0 + lane < m.nfall)
         b.q[i0 + lane] = falloff_rate(m, b.C, b.g, i0 + lane, T, logT, invT, lnPf, Ctot);
-#if KIN_WARP_PAIRED_RATES
-    for (int i0 = m.nfall; i0 < m.nr; i0 += 2 * L) {
-      const int ia = i0 + lane, ib = i0 + L + lane;
-      const int ca = ia < m.nr ? ia : m.nr - 1, cb = ib < m.nr ? ib : m.nr - 1;
-      const double qa = elem_rate(m, b.C, b.g, ca, logT, invT, lnPf);
-      const double qb = elem_rate(m, b.C, b.g, cb, logT, invT, lnPf);
-      if (ia < m.nr) b.q[ia] = qa;
-      if (ib < m.nr) b.q[ib] = qb;
-    }
-#else
     for (int i0 = m.nfall; i0 < m.nr; i0 += L)
       if (i0 + lane < m.nr) b.q[i0 + lane] = elem_rate(m, b.C, b.g, i0 + lane, logT, invT, lnPf);
-#endif
   }
   const int nr_with_jac = wantJ ? m.nr : 0;
   for (int i0 = 0; i0 < nr_with_jac; i0 += L) {
