@@ -151,14 +151,26 @@ __device__ __forceinline__ void bind_scratch(Work<MAXN, LT> &w, const KernelArgs
 #endif
 }
 
-// Resident 64-thread blocks per SM that a PLAIN kernel's registers allow.  A
-// batch that fills the chip takes KIN_THREAD_MIN_BLOCKS (48 registers: hiding
-// latency is worth more than spills); one that leaves SMs with fewer blocks
-// than that anyway takes the registers they leave free (168, 96 or 72), which
-// spill less.  Ordered mixed H2 states, dt = 1e-4 s, ms, with 48 registers and
-// with the free ones: FP64 50021: 315, 304, 80000: 793, 515, 131072: 1153, 896;
-// FP32 50021: 240, 222, 80000: 525, 364, 131072: 772, 617.
+// Resident 64-thread blocks per SM that a PLAIN kernel's registers allow.  What
+// bounds a batch is the FP64 unit, which a few warps per sub-partition keep
+// busy, the spills that fewer registers cost, and the last wave's tail.  A
+// batch of many waves takes KIN_THREAD_MIN_BLOCKS (48 registers: the tail is
+// short, hiding the spills' latency pays); one of a wave or two takes the
+// variant (168, 96 or 72 registers) that was fastest for its blocks per SM.
+// Ordered mixed H2 states, ms with 6, 10, 14 and 20 blocks per SM, FP64 at
+// dt = 1e-6 s, then FP32 matrices at 1e-4 s:
+//    50021 ( 6 blocks per SM)  203 210 211 214    223 230 236 239
+//    80000 ( 9)                323 287 338 400    397 365 414 504
+//   131072 (14)                471 491 523 705    614 578 644 735
+//   160000 (17)                    568 607 739        619 675 776
+//   200000 (21)                712 690 687 765    847 879 743 799
+//   220000 (23)                    769 737 830        919 854 839
+//  1048576 (108), FP32 only                      3986 3758 3565 3337
+// and in input order with 10, 14 and 20:
+//   160000                         683 791 917        662 683 827
+//   180000 (19)                    905 831 942        820 746 836
 constexpr int PLAIN_BLOCKS_FEW = 6, PLAIN_BLOCKS_MID = 10, PLAIN_BLOCKS_MANY = 14;
+constexpr int PLAIN_USE_FEW = 6, PLAIN_USE_MID = 17, PLAIN_USE_MANY = 21;  // up to, per SM
 
 template <int MAXN, typename LT, bool FDJ, int MINB>
 __global__ void __launch_bounds__(64, MINB) k_integrate_plain(KernelArgs a) {
@@ -543,11 +555,11 @@ int launch_t(const KernelArgs &a, const kin_options &o, cudaStream_t st, int sms
     void (*kern)(KernelArgs) = k_integrate_plain<MAXN, LT, FDJ, KIN_THREAD_MIN_BLOCKS>;
     if constexpr (MAXN <= 16 && !FDJ) {
       const int64_t per_sm = (a.rp.n + 64ll * sms - 1) / (64ll * sms);
-      if (per_sm <= PLAIN_BLOCKS_FEW)
+      if (per_sm <= PLAIN_USE_FEW)
         kern = k_integrate_plain<MAXN, LT, FDJ, PLAIN_BLOCKS_FEW>;
-      else if (per_sm <= PLAIN_BLOCKS_MID)
+      else if (per_sm <= PLAIN_USE_MID)
         kern = k_integrate_plain<MAXN, LT, FDJ, PLAIN_BLOCKS_MID>;
-      else if (per_sm <= PLAIN_BLOCKS_MANY)
+      else if (per_sm <= PLAIN_USE_MANY)
         kern = k_integrate_plain<MAXN, LT, FDJ, PLAIN_BLOCKS_MANY>;
     }
     KIN_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
