@@ -381,7 +381,7 @@ def config3_leg(stream, form="massfrac", n=0):
     tot = mg.stats()
     ops = op_model(mech, form)
     f64, f32 = algorithmic_flops(tot, ops, True) if ops else (None, None)
-    kernel = "k_integrate_conc<32, float>" if conc else "k_integrate_lanes<32, float>"
+    kernel = "k_integrate_conc<float>" if conc else "k_integrate_team<float>"
     rec = {"workload": "ch4_2p18", "states": st.n, "species": mech.ns, "reactions": mech.nr,
            "dt": 1e-4, "layout": "warp", "lanes": 32, "newton_matrices": "fp32",
            "form": "concentration-based, sparse LU" if conc else "mass fractions, dense LU",
