@@ -15,7 +15,7 @@
 // the complex linear algebra on different warps, the complex substitution's
 // real and imaginary parts on different lanes; everything lives in shared
 // memory.  Measured (FP64, dt = 1e-6 s): 33 states 123 -> 9.3 ms, 1024 states
-// 153 -> 23 ms.  What is left on one state: 35 % chemistry (the Troe branch
+// 153 -> 20.7 ms.  What is left on one state: 35 % chemistry (the Troe branch
 // and the logarithms), 25 % substitutions (78 dependent terms), 15 %
 // factorisations, the rest scalar control and norms.
 //
