@@ -880,7 +880,7 @@ __global__ void __launch_bounds__(TEAM_MAX *TEAM_NT, 1)
     return;
   }
   f.v[0] = f.v[1] = 0.0;
-  double *f0s = t.js + 3 * wt * t.nv, *ys = f0s + t.nv, *sc = ys + t.nv;  // eight vectors + 2 nr
+  double *f0s = t.fd(wt), *ys = f0s + t.nv, *sc = ys + t.nv;
   for (int64_t i = first * TEAM_WARPS + wt; i < n; i += step * TEAM_WARPS) {
     load(y, i, v);
     (void)team_rhs<>(m, h, t.C(wt), t.g(wt), t.q(wt), a.P[i], v, f);
@@ -922,9 +922,7 @@ __global__ void __launch_bounds__(TEAM_MAX *TEAM_NT, 1)
 template <int WHAT>
 static bool chem_on_teams(kin_mech *m, double h, const double *scal, const double *y,
                           const double *P, int64_t n, double *out, cudaStream_t st, int &rc) {
-  // three vectors per warp in the eight vectors and two reaction lists of the
-  // Jacobian's scratch
-  if (m->L.ns <= 16 || m->L.ns > 63 || 2 * m->L.nr < team_nv(m->L.ns)) return false;
+  if (m->L.ns <= 16 || m->L.ns > 63 || !team_fd_fits(m->L.ns)) return false;
   int dev = 0, sms = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev != m->device ||
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {

@@ -162,13 +162,26 @@ struct TeamBuf {
   LT *d1;            // reciprocals of E1's pivots (FP64)
   unsigned char *p1, *p2;  // row sources after all exchanges (p2: bit 7 Smith's case)
   TeamCtl *ctl;
-  __device__ __forceinline__ double *C(int w) const { return w ? w12 + (w - 1) * wstride : w0; }
+  __host__ __device__ __forceinline__ double *C(int w) const {
+    return w ? w12 + (w - 1) * wstride : w0;
+  }
   __device__ __forceinline__ double *g(int w) const { return C(w) + nv; }
   __device__ __forceinline__ double *q(int w) const { return C(w) + 2 * nv; }
+  // warp w's vectors of a difference Jacobian (team_fd_doubles)
+  __host__ __device__ __forceinline__ double *fd(int w) const { return Jd + 3 * w * nv; }
 };
 
 __host__ __device__ inline int team_nv(int ns) { return (ns + 2) & ~1; }
 __host__ __device__ inline int team_ld(int N) { return N | 1; }
+// Three vectors per warp for a state per warp's difference Jacobian, in the
+// assembly matrix's area (N x team_ld doubles), which that kernel leaves alone:
+// the other areas are its warps' live rate buffers.  They fit from 10 species on.
+__host__ __device__ inline size_t team_fd_doubles(int ns) {
+  return 3 * TEAM_WARPS * (size_t)team_nv(ns);
+}
+__host__ __device__ inline bool team_fd_fits(int ns) {
+  return team_fd_doubles(ns) <= (size_t)ns * team_ld(ns);
+}
 // Jacobian scratch in doubles: eight species vectors, two reaction vectors
 // and the derivatives by slot and by collision partner
 __host__ __device__ inline size_t team_js_doubles(const MechLayout &L) {
@@ -188,7 +201,7 @@ __host__ __device__ inline size_t team_bytes(const MechLayout &L, int N, size_t 
 }
 
 template <typename LT>
-__device__ TeamBuf<LT> carve_team(const MechLayout &L, unsigned char *p, int team, int N,
+__host__ __device__ inline TeamBuf<LT> carve_team(const MechLayout &L, unsigned char *p, int team, int N,
                                   unsigned char *slot) {
   const int ns = L.ns, nr = L.nr;
   TeamBuf<LT> t;
