@@ -941,8 +941,7 @@ static bool chem_on_teams(kin_mech *m, double h, const double *scal, const doubl
   if (!team_shape(a, a.L.ns, sizeof(float), sms, g)) return false;
   auto kern = k_team_chem<WHAT>;
   rc = KIN_OK;
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g.smem) !=
-      cudaSuccess) {
+  if (open_smem(kern) != cudaSuccess) {
     (void)cudaGetLastError();
     rc = KIN_ERR_CUDA;
     return true;
@@ -963,10 +962,10 @@ extern "C" int kin_rhs(kin_mech *m, const double *y, const double *P, int64_t n,
   const int block = 64;
   const unsigned grid = (unsigned)((n + block - 1) / block);
   if (m->L.ns <= 16) {
-    KIN_CUDA_TRY(cudaFuncSetAttribute(k_rhs<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    KIN_CUDA_TRY(open_smem(k_rhs<16>));
     k_rhs<16><<<grid, block, sm, st>>>(m->L, m->d_tab, m->d_itab, y, P, n, f);
   } else {
-    KIN_CUDA_TRY(cudaFuncSetAttribute(k_rhs<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    KIN_CUDA_TRY(open_smem(k_rhs<64>));
     k_rhs<64><<<grid, block, sm, st>>>(m->L, m->d_tab, m->d_itab, y, P, n, f);
   }
   KIN_CUDA_TRY(cudaGetLastError());
@@ -986,10 +985,10 @@ extern "C" int kin_jacobian(kin_mech *m, const double *y, const double *P, int64
   const int block = 64;
   const unsigned grid = (unsigned)((n + block - 1) / block);
   if (m->L.ns <= 16) {
-    KIN_CUDA_TRY(cudaFuncSetAttribute(k_jac<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    KIN_CUDA_TRY(open_smem(k_jac<16>));
     k_jac<16><<<grid, block, sm, st>>>(m->L, m->d_tab, m->d_itab, y, P, n, fd, h, scal, J);
   } else {
-    KIN_CUDA_TRY(cudaFuncSetAttribute(k_jac<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    KIN_CUDA_TRY(open_smem(k_jac<64>));
     k_jac<64><<<grid, block, sm, st>>>(m->L, m->d_tab, m->d_itab, y, P, n, fd, h, scal, J);
   }
   KIN_CUDA_TRY(cudaGetLastError());

@@ -263,7 +263,7 @@ int launch_conc(ConcArgs ca, cudaStream_t st, int sms) {
   TeamLaunch g;
   if (!team_shape(a, ca.N, sizeof(LT), sms, g)) return KIN_ERR_UNSUPPORTED;
   auto kern = k_integrate_conc<LT>;
-  KIN_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g.smem));
+  KIN_CUDA_TRY(open_smem(kern));
   kern<<<g.grid, g.threads, g.smem, st>>>(ca);
   KIN_CUDA_TRY(cudaGetLastError());
   return KIN_OK;

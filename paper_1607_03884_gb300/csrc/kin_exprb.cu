@@ -710,7 +710,7 @@ __global__ void k_exprb_chem(MechLayout L, const double *tab, const int *itab,
 // whether the tables are staged, and their bytes; false when not even one
 // warp's buffers fit
 bool xshape(const MechLayout &L, int &hot_smem, size_t &fixed) {
-  const size_t budget = 227 * 1024, hot = hot_offsets(L).bytes, per = xwarp_bytes(L);
+  const size_t budget = BLOCK_SMEM, hot = hot_offsets(L).bytes, per = xwarp_bytes(L);
   if (per > budget) return false;
   hot_smem = hot + per <= budget;
   fixed = hot_smem ? hot : 0;
@@ -821,13 +821,13 @@ extern "C" int kin_integrate_exprb(kin_exprb *x, double *Y, double *T, const dou
   a.hot = x->d_hot;
   size_t fixed = 0;
   if (!xshape(x->L, a.hot_smem, fixed)) return KIN_ERR_UNSUPPORTED;
-  const size_t budget = 227 * 1024, per = xwarp_bytes(x->L);
+  const size_t budget = BLOCK_SMEM, per = xwarp_bytes(x->L);
   auto kern = k_integrate_exprb;
+  KIN_CUDA_TRY(open_smem(kern));
   int warps = 0, per_sm = 0;
   for (int wp = 8; wp >= 1; wp >>= 1) {
     const size_t smw = fixed + (size_t)wp * per;
     if (smw > budget) continue;
-    KIN_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smw));
     int nb = 0;
     KIN_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, 32 * wp, smw));
     if (nb * wp > per_sm * warps) {
@@ -837,7 +837,6 @@ extern "C" int kin_integrate_exprb(kin_exprb *x, double *Y, double *T, const dou
   }
   if (warps < 1 || per_sm < 1) return KIN_ERR_UNSUPPORTED;
   const size_t sm = fixed + (size_t)warps * per;
-  KIN_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
   int64_t grid = (int64_t)sms * per_sm;
   const int64_t need = (n + warps - 1) / warps;
   if (grid > need) grid = need;
@@ -874,8 +873,7 @@ extern "C" int kin_exprb_chem(kin_exprb *x, const double *y, const double *P, in
   size_t fixed = 0;
   if (!xshape(x->L, hot_smem, fixed)) return KIN_ERR_UNSUPPORTED;
   const size_t sm = fixed + xwarp_bytes(x->L);
-  KIN_CUDA_TRY(cudaFuncSetAttribute(k_exprb_chem, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)sm));
+  KIN_CUDA_TRY(open_smem(k_exprb_chem));
   const int64_t grid = n < x->slots ? n : x->slots;
   k_exprb_chem<<<(unsigned)grid, XL, sm, (cudaStream_t)stream>>>(
       x->L, x->d_tab, x->d_itab, x->d_hot, hot_smem, y, P, n, f, f_rates, J, x->d_scratch,

@@ -21,6 +21,16 @@ namespace kin {
     }                                                                         \
   } while (0)
 
+// Shared memory a block may hold, and a kernel opened to it.  The limit is an
+// attribute of the kernel in the whole process: set to what a call needs,
+// another thread's smaller call could lower it between this call's setting and
+// its launch, which is then refused.  So it is always set to the whole.
+constexpr size_t BLOCK_SMEM = 227 * 1024;
+template <typename K>
+inline cudaError_t open_smem(K *kern) {
+  return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)BLOCK_SMEM);
+}
+
 __host__ __device__ inline size_t smem_bytes(const MechLayout &L) {
   return sizeof(double) * (size_t)L.nd + sizeof(int) * (size_t)L.ni;
 }
@@ -463,7 +473,7 @@ struct TeamLaunch {
 // species vectors.  (Only some 2900 reactions of six slots that change no
 // species at all would not; they are refused.)
 inline bool team_shape(KernelArgs &a, int N, size_t lt, int sms, TeamLaunch &g) {
-  const size_t budget = 227 * 1024, tb = team_bytes(a.L, N, lt), hot = hot_offsets(a.L).bytes;
+  const size_t budget = BLOCK_SMEM, tb = team_bytes(a.L, N, lt), hot = hot_offsets(a.L).bytes;
   if (!a.hot || tb > budget) return false;
   a.hot_smem = hot + tb <= budget;
   const size_t fixed = a.hot_smem ? hot : 0;
@@ -485,7 +495,7 @@ int launch_team(KernelArgs a, cudaStream_t st, int sms) {
   TeamLaunch g;
   if (!team_shape(a, a.L.ns, sizeof(LT), sms, g)) return KIN_ERR_UNSUPPORTED;
   auto kern = k_integrate_team<LT, FDJ>;
-  KIN_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g.smem));
+  KIN_CUDA_TRY(open_smem(kern));
   kern<<<g.grid, g.threads, g.smem, st>>>(a);
   KIN_CUDA_TRY(cudaGetLastError());
   return KIN_OK;
@@ -496,14 +506,14 @@ int launch_lanes(const KernelArgs &a, cudaStream_t st, int sms) {
   using G = Grp<L>;
   if (a.L.ns >= G::CAP) return KIN_ERR_UNSUPPORTED;
   if (!a.gscratch || a.gslots < 1) return KIN_ERR_UNSUPPORTED;
-  const size_t budget = 227 * 1024;
+  const size_t budget = BLOCK_SMEM;
   auto kern = k_integrate_lanes<L, LT, FDJ>;
+  KIN_CUDA_TRY(open_smem(kern));
   // the block size (1 to 8 warps) that keeps the most warps resident per SM
   int warps = 0, per_sm = 0;
   for (int w = 8; w >= 1; w >>= 1) {
     const size_t smw = lanes_smem_bytes(a.L, L, sizeof(LT), w);
     if (smw > budget) continue;
-    KIN_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smw));
     int b = 0;
     KIN_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, kern, 32 * w, smw));
     if (b * w > per_sm * warps) {
@@ -513,7 +523,6 @@ int launch_lanes(const KernelArgs &a, cudaStream_t st, int sms) {
   }
   if (warps < 1 || per_sm < 1) return KIN_ERR_UNSUPPORTED;
   const size_t sm = lanes_smem_bytes(a.L, L, sizeof(LT), warps);
-  KIN_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
   int64_t grid = (int64_t)sms * per_sm;
   const int64_t per_block = (int64_t)warps * (32 / L);
   const int64_t need = (a.rp.n + per_block - 1) / per_block;
@@ -545,7 +554,7 @@ int launch_t(const KernelArgs &a, const kin_options &o, cudaStream_t st, int sms
     if (plain && a.rp.n <= coop_max_n(sizeof(LT)) &&
         smc <= COOP_MAX_SMEM) {
       auto kern = k_integrate_coop<LT, FDJ>;
-      KIN_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smc));
+      KIN_CUDA_TRY(open_smem(kern));
       kern<<<(unsigned)a.rp.n, COOP_NT, smc, st>>>(a);
       KIN_CUDA_TRY(cudaGetLastError());
       return KIN_OK;

@@ -171,12 +171,10 @@ int launch_order(const MechLayout &L, const double *tab, const int *itab, const 
     const int block = 64;
     const unsigned grid = (unsigned)((n + block - 1) / block);
     if (L.ns <= 16) {
-      KIN_CUDA_TRY(cudaFuncSetAttribute(k_order_key<16>,
-                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+      KIN_CUDA_TRY(open_smem(k_order_key<16>));
       k_order_key<16><<<grid, block, sm, st>>>(L, tab, itab, Y, T, P, n, rtol, atol, key);
     } else {
-      KIN_CUDA_TRY(cudaFuncSetAttribute(k_order_key<64>,
-                                        cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+      KIN_CUDA_TRY(open_smem(k_order_key<64>));
       k_order_key<64><<<grid, block, sm, st>>>(L, tab, itab, Y, T, P, n, rtol, atol, key);
     }
     KIN_CUDA_TRY(cudaGetLastError());
