@@ -551,7 +551,7 @@ int launch_t(const KernelArgs &a, const kin_options &o, cudaStream_t st, int sms
   const int carve = KIN_THREAD_CARVEOUT;  // percent of the unified L1 given to shared memory
   if constexpr (MAXN <= COOP_CAP) {
     const size_t smc = coop_smem_bytes<LT>(a.L.nr);
-    if (plain && a.rp.n <= coop_max_n(sizeof(LT)) &&
+    if (plain && a.rp.n > 0 && a.rp.n <= coop_max_n(sizeof(LT)) &&
         smc <= COOP_MAX_SMEM) {
       auto kern = k_integrate_coop<LT, FDJ>;
       KIN_CUDA_TRY(open_smem(kern));
@@ -561,20 +561,24 @@ int launch_t(const KernelArgs &a, const kin_options &o, cudaStream_t st, int sms
     }
   }
   if (plain) {
+    // the variant with the fewest registers has the largest frame; an empty
+    // batch (reserve_frames) runs one idle block of it
     void (*kern)(KernelArgs) = k_integrate_plain<MAXN, LT, FDJ, KIN_THREAD_MIN_BLOCKS>;
     if constexpr (MAXN <= 16 && !FDJ) {
       const int64_t per_sm = (a.rp.n + 64ll * sms - 1) / (64ll * sms);
-      if (per_sm <= PLAIN_USE_FEW)
-        kern = k_integrate_plain<MAXN, LT, FDJ, PLAIN_BLOCKS_FEW>;
-      else if (per_sm <= PLAIN_USE_MID)
-        kern = k_integrate_plain<MAXN, LT, FDJ, PLAIN_BLOCKS_MID>;
-      else if (per_sm <= PLAIN_USE_MANY)
-        kern = k_integrate_plain<MAXN, LT, FDJ, PLAIN_BLOCKS_MANY>;
+      if (per_sm > 0) {
+        if (per_sm <= PLAIN_USE_FEW)
+          kern = k_integrate_plain<MAXN, LT, FDJ, PLAIN_BLOCKS_FEW>;
+        else if (per_sm <= PLAIN_USE_MID)
+          kern = k_integrate_plain<MAXN, LT, FDJ, PLAIN_BLOCKS_MID>;
+        else if (per_sm <= PLAIN_USE_MANY)
+          kern = k_integrate_plain<MAXN, LT, FDJ, PLAIN_BLOCKS_MANY>;
+      }
     }
     KIN_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
     KIN_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, carve));
     const int64_t grid = (a.rp.n + block - 1) / block;
-    kern<<<(unsigned)grid, block, sm, st>>>(a);
+    kern<<<grid > 0 ? (unsigned)grid : 1u, block, sm, st>>>(a);
   } else {
     auto kern = k_integrate_queue<MAXN, LT, FDJ>;
     KIN_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));

@@ -37,6 +37,7 @@ static __device__ __align__(256) unsigned char g_scratch[KIN_STATIC_SCRATCH_BYTE
 
 std::mutex g_mu;
 unsigned char *g_addr[64];  // device address of g_scratch per device (set-up done when non-null)
+bool g_framed[64];          // reserve_frames done
 
 int scratch_address(int dev, unsigned char **out) {
   std::lock_guard<std::mutex> lk(g_mu);
@@ -52,6 +53,22 @@ int scratch_address(int dev, unsigned char **out) {
   }
   *out = g_addr[dev];
   return KIN_OK;
+}
+
+// A mechanism of up to COOP_CAP species runs a small batch on a kernel without
+// a per-thread frame and a large one on kernels with some 13 KB a thread, for
+// which the driver reserves local memory at their first launch.  The first
+// call on a device has the driver reserve it whatever its batch: an empty
+// launch of the kernel with the largest frame.
+int reserve_frames(int dev, const KernelArgs &args, const kin_options &o, cudaStream_t st,
+                   int sms) {
+  std::lock_guard<std::mutex> lk(g_mu);
+  if (args.L.ns > COOP_CAP || g_framed[dev]) return KIN_OK;
+  KernelArgs a = args;
+  a.rp.n = 0;
+  const int rc = launch_dispatch(a, o, st, sms);
+  if (!rc) g_framed[dev] = true;
+  return rc;
 }
 
 }  // namespace
@@ -131,5 +148,6 @@ extern "C" int kin_integrate_static(const kin_mech_desc *desc, double *Y, double
   a.gslots = 0;
   a.hot = nullptr;
   a.hot_smem = 0;
+  if ((rc = reserve_frames(dev, a, o, st, sms))) return rc;
   return launch_dispatch(a, o, st, sms);
 }
