@@ -1120,24 +1120,37 @@ static bool mlp_maps(kin_mlp *n) {
   return ok;
 }
 
+template <typename X>
+static void drop(X *&p) {
+  cudaFree(p);
+  p = nullptr;
+}
+
+// the activations' buffers and what describes them; the pointers are cleared,
+// so that a handle whose growth failed is neither read nor freed again
+static void mlp_release(kin_mlp *n) {
+  drop(n->xg);
+  drop(n->tg);
+  drop(n->xf);
+  drop(n->xb);
+  drop(n->C);
+  drop(n->g);
+  drop(n->dH);
+  drop(n->gb);
+  drop(n->gb2);
+  for (int l = 0; l < LAYERS; ++l) {
+    drop(n->a[l]);
+    drop(n->hf[l]);
+    drop(n->hb[l]);
+  }
+  n->y = nullptr;
+  n->cap = 0;
+  n->maps = false;
+}
+
 static int mlp_reserve(kin_mlp *n, int64_t rows) {
   if (rows <= n->cap) return KIN_OK;
-  cudaFree(n->xg);
-  cudaFree(n->tg);
-  n->xg = n->tg = nullptr;
-  cudaFree(n->xf);
-  cudaFree(n->xb);
-  cudaFree(n->C);
-  cudaFree(n->g);
-  cudaFree(n->dH);
-  cudaFree(n->gb);
-  cudaFree(n->gb2);
-  for (int l = 0; l < LAYERS; ++l) {
-    cudaFree(n->a[l]);
-    cudaFree(n->hf[l]);
-    cudaFree(n->hb[l]);
-  }
-  n->cap = 0;
+  mlp_release(n);
   const int64_t wmax = n->width > n->doutp ? n->width : n->doutp;
   KIN_CUDA_TRY(cudaMalloc(&n->xg, sizeof(float) * rows * n->din));
   KIN_CUDA_TRY(cudaMalloc(&n->tg, sizeof(float) * rows * n->dout));
@@ -1435,20 +1448,7 @@ extern "C" void kin_mlp_destroy(kin_mlp *n) {
   cudaFree(n->ws);
   cudaFree(n->loss);
   cudaFree(n->err);
-  cudaFree(n->xg);
-  cudaFree(n->tg);
-  cudaFree(n->xf);
-  cudaFree(n->xb);
-  cudaFree(n->C);
-  cudaFree(n->g);
-  cudaFree(n->dH);
-  cudaFree(n->gb);
-  cudaFree(n->gb2);
-  for (int l = 0; l < LAYERS; ++l) {
-    cudaFree(n->a[l]);
-    cudaFree(n->hf[l]);
-    cudaFree(n->hb[l]);
-  }
+  mlp_release(n);
   delete n;
 }
 
