@@ -26,3 +26,21 @@ def test_a_handle_survives_a_batch_that_does_not_fit(width):
         assert rc == kin.KIN_ERR_NOMEM
     net.forward(X, Y[1])
     assert torch.equal(*Y)
+
+
+def test_a_first_batch_allocates_what_its_path_uses():
+    """Width 256, 56 inputs, 160 outputs, per row: BF16 input (64) and
+    activations (3 x 256 + 160), FP32 pre-activations (3 x 256), two gradient
+    pairs of 256 in both types."""
+    rows = 1 << 18
+    net = kin.MLP(56, 256, 160)
+    X = torch.zeros((rows, 56), device="cuda")
+    Y = torch.zeros((rows, 160), device="cuda")
+    net.forward(X[:1], Y[:1])
+    torch.cuda.synchronize()
+    before = torch.cuda.mem_get_info()[0]
+    net.forward(X, Y)
+    torch.cuda.synchronize()
+    per_row = 2 * (64 + 3 * 256 + 160) + 4 * 3 * 256 + 2 * (4 + 2) * 256
+    # each of twelve allocations may round up to a 2 MiB page
+    assert before - torch.cuda.mem_get_info()[0] <= rows * per_row + (12 << 21)
