@@ -1279,6 +1279,7 @@ __device__ __forceinline__ void team_exec(int cmd, int wt, const Form &f) {
 // drivers' buffer argument stays unused: the matrices are the team's).
 template <typename LT, class Form>
 struct TeamSys {
+  static constexpr int POINTS = TEAM_WARPS;
   using WV = WVecT<2>;
   const Form &f;
   __device__ __forceinline__ int n() const { return f.n(); }

@@ -797,7 +797,8 @@ __device__ int warp_factor(int N, const WarpBuf<LT> &b, double h) {
 
 // The system a group integrates, as a policy of the step drivers below: its
 // size n(), the absolute tolerance's factor per element atol_w(), right-hand
-// side (and Jacobian) chem(), the right-hand sides at three points chem3(),
+// side (and Jacobian) chem(), the right-hand sides at three points chem3() and
+// how many points those take the time of one (POINTS, 1 or 3),
 // factorisation of E1 and E2 factor(), the two solves (and both of a Newton
 // iteration, solve_both()), and where the stored Jacobian keeps entry (i, j),
 // jat().  MassFracSys is the mass-fraction reactor
@@ -805,6 +806,7 @@ __device__ int warp_factor(int N, const WarpBuf<LT> &b, double h) {
 // concentration-based form with a sparse LU.
 template <int L, typename LT>
 struct MassFracSys {
+  static constexpr int POINTS = 1;
   using WV = WVecT<Grp<L>::WR>;
   const MechView *m;
   __device__ __forceinline__ int n() const { return m->ns; }
@@ -994,11 +996,13 @@ __device__ bool warp_step_sys(const Sys &sys, const WarpBuf<LT> &b, double P,
         const double fn = wrms_w<L>(N, w.f0, w.scal);
         const double mininc =
             (fn != 0.0) ? 1000.0 * fabs(s.h) * 2.220446049250313e-16 * N * fn : 1.0;
-        for (int j0 = 0; j0 < N; j0 += 3) {  // three columns at a time
-          WVecT<WR> u[3], fj[3];
-          double inc[3];
+        // as many columns at a time as the system evaluates side by side
+        constexpr int Q = Sys::POINTS;
+        for (int j0 = 0; j0 < N; j0 += Q) {
+          WVecT<WR> u[Q], fj[Q];
+          double inc[Q];
 #pragma unroll
-          for (int q = 0; q < 3; ++q) {
+          for (int q = 0; q < Q; ++q) {
             const int j = j0 + q < N ? j0 + q : N - 1;
             const double yj = elem<L>(w.y, j);
             const double sj = elem<L>(w.scal, j);
@@ -1007,9 +1011,12 @@ __device__ bool warp_step_sys(const Sys &sys, const WarpBuf<LT> &b, double P,
             for (int r = 0; r < WR; ++r) u[q].v[r] = w.y.v[r];
             if (lane == (j & (L - 1))) slot_set<WR>(u[q], j / L, yj + inc[q]);
           }
-          rc |= sys.chem3(b, P, u[0], u[1], u[2], fj[0], fj[1], fj[2]);
+          if constexpr (Q == 3)
+            rc |= sys.chem3(b, P, u[0], u[1], u[2], fj[0], fj[1], fj[2]);
+          else
+            rc |= sys.chem(b, P, u[0], fj[0], false);
 #pragma unroll
-          for (int q = 0; q < 3; ++q)
+          for (int q = 0; q < Q; ++q)
 #pragma unroll
             for (int r = 0; r < WR; ++r) {
               const int i = lane + L * r;
