@@ -420,7 +420,12 @@ struct Coop {
     src = __shfl_sync(0xffffffffu, src, to);
   }
 
-  __device__ static void pair_sync() { asm volatile("bar.sync 1, 64;" ::: "memory"); }
+  // warps 1 and 2; bar.sync takes converged warps only, and lanes arrive here
+  // from loops of different lengths
+  __device__ static void pair_sync() {
+    __syncwarp();
+    asm volatile("bar.sync 1, 64;" ::: "memory");
+  }
 
   // lu_cplx on warps 1 and 2: both find the pivot, a lane's row is its lane
   // modulo 16, its columns every fourth.  The multipliers' real parts are
