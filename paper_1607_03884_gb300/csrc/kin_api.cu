@@ -842,6 +842,35 @@ extern "C" int kin_order_states(kin_mech *m, const double *Y, const double *T, c
 // ---------------------------------------------------------------------------
 enum { CHEM_RHS = 0, CHEM_JAC, CHEM_FD };
 
+// Batches beyond this many states go to the thread kernels.  A team's or warp's
+// time grows with the batch and fills its lanes in part (17 species, reactions
+// in rounds of 32); a thread's is flat, the chain of a state's operations, until
+// every sub-partition has a warp of 32 states, and grows with them from there.
+// So the lines cross later for longer chains, about in proportion to nr (80 +
+// ns) for right-hand sides and difference Jacobians and 2.2 times that for
+// analytical ones; with long ones the threads' frames leave the caches, and
+// teams stay ahead much longer or for good.  The CH4 mechanism and subsets of
+// its species, ms, teams against threads:
+//               right-hand side          difference            analytical
+//   17 species   2500  0.10   0.12    2500   1.6   2.0     5000  0.36   0.46
+//   29 reactions 5000  0.14   0.12    5000   2.4   2.0    10000  0.66   0.51
+//               40000  0.90   0.22   40000  17     4.1   100000  6.2    2.0
+//   24           5000  0.16   0.20    5000   3.6   4.8    15000  1.2    1.4
+//   59           7500  0.25   0.20    7500   6.0   4.8    20000  1.6    1.5
+//   32          10000  0.34   0.48   10000  11    16      20000  2.2    3.2
+//   116         20000  0.59   0.53   20000  20    17      40000  4.4    3.8
+//   44          20000  0.73   0.78   20000  33    36      40000  6.2    6.5
+//   179         30000  1.1    0.87   30000  51    39     100000 15.5   13.5
+//   53          40000  1.8    2.4    40000 101   132      40000  8.6   18.2
+//   325        100000  4.6    4.8    60000 151   190     100000 21.4   37.9
+// The two kernels round in different orders: a state's last bits depend on the
+// side of the line.
+static int64_t chem_team_max(const MechLayout &L, int what) {
+  const int64_t chain = (int64_t)L.nr * (80 + L.ns);
+  if (what == CHEM_JAC) return L.nr > 200 ? INT64_MAX : chain * 11 / 5;
+  return L.nr > 256 ? 2 * chain : chain;
+}
+
 template <int WHAT>
 __global__ void __launch_bounds__(TEAM_MAX *TEAM_NT, 1)
     k_team_chem(KernelArgs a, double h_step, const double *scal, const double *y, double *out) {
@@ -918,11 +947,13 @@ __global__ void __launch_bounds__(TEAM_MAX *TEAM_NT, 1)
   }
 }
 
-// false when the thread kernel has to serve (small mechanisms; no team fits)
+// false when the thread kernel has to serve (small mechanisms, large batches; no
+// team fits)
 template <int WHAT>
 static bool chem_on_teams(kin_mech *m, double h, const double *scal, const double *y,
                           const double *P, int64_t n, double *out, cudaStream_t st, int &rc) {
   if (m->L.ns <= 16 || m->L.ns > 63 || !team_fd_fits(m->L.ns)) return false;
+  if (n > chem_team_max(m->L, WHAT)) return false;
   int dev = 0, sms = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev != m->device ||
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {

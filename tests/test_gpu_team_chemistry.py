@@ -1,7 +1,8 @@
 """kin_rhs and both kinds of kin_jacobian on teams of warps at the species
 counts where their shared memory is tightest (17, 18), where the two register
 slots meet (32, 33) and at the largest (63), against the oracle, for batches
-that leave a team's warps idle (1), fill one team (3) and fill many (500)."""
+that leave a team's warps idle (1), fill one team (3) and fill many (500), and
+on both sides of the lines beyond which the thread kernels serve."""
 import numpy as np
 import pytest
 
@@ -32,9 +33,7 @@ def _jac(mg, y, P, scal=None):
     return J.cpu().numpy().reshape(N, N, n)
 
 
-@pytest.mark.parametrize("n", [1, 3, 500])
-@pytest.mark.parametrize("ns", [17, 18, 19, 32, 33, 63])
-def test_chemistry_against_the_oracle(ns, n):
+def _against_the_oracle(ns, n):
     h2 = synth.make_mechanism("h2")
     m = _with_spectators(h2, ns)
     st = _states(h2, n, ns, 40 + ns)
@@ -49,21 +48,38 @@ def test_chemistry_against_the_oracle(ns, n):
         colmax = np.abs(Jo).max(axis=0) + 1e-300
         assert np.max(np.abs(J[:, :, i] - Jo) / colmax) < 1e-9, i
         # difference quotients with the same increments differ by the two
-        # sides' right-hand sides at the two points, over the increment
+        # sides' right-hand sides at the two points, over the increment; the
+        # device's are taken in a batch of the same size, by the same kernel
         Jd, rc = O.jac_fd(om, P, yi, fo, H, scal[:, i])
         assert rc == 0
         fn = np.sqrt(np.mean((fo / scal[:, i]) ** 2))
         inc = np.maximum(np.sqrt(eps) * np.abs(yi), 1000.0 * H * eps * ns * fn * scal[:, i])
         yp = np.repeat(yi[:, None], ns + 1, axis=1)
         yp[np.arange(ns), 1 + np.arange(ns)] += inc
-        df = np.abs(_rhs(mg, yp, np.full(ns + 1, P))
+        cols = np.arange(max(n, ns + 1)) % (ns + 1)
+        df = np.abs(_rhs(mg, yp[:, cols], np.full(cols.size, P))[:, :ns + 1]
                     - np.stack([O.rhs(om, P, yp[:, c])[0] for c in range(ns + 1)], axis=1))
         bound = (1e-9 * (np.abs(Jd).max(axis=0) + 1e-300)[None, :]
                  + 1.01 * (df[:, 1:] + df[:, :1]) / inc[None, :] + 1e-300)
         assert np.all(np.abs(Jfd[:, :, i] - Jd) <= bound), i
+    return mg, st, y, scal, f, J, Jfd
+
+
+@pytest.mark.parametrize("n", [1, 3, 500])
+@pytest.mark.parametrize("ns", [17, 18, 19, 32, 33, 63])
+def test_chemistry_against_the_oracle(ns, n):
+    mg, st, y, scal, f, J, Jfd = _against_the_oracle(ns, n)
     # and a state's results do not depend on the batch it comes in
     for i in sorted({0, n // 3, n - 1}):
         s = slice(i, i + 1)
         np.testing.assert_array_equal(f[:, s], _rhs(mg, y[:, s], st.P[s]))
         np.testing.assert_array_equal(J[:, :, s], _jac(mg, y[:, s], st.P[s]))
         np.testing.assert_array_equal(Jfd[:, :, s], _jac(mg, y[:, s], st.P[s], scal[:, s]))
+
+
+@pytest.mark.parametrize("ns", [17, 24, 63])
+@pytest.mark.parametrize("kind", ["rhs and differences", "analytical"])
+@pytest.mark.parametrize("over", [0, 1])
+def test_both_sides_of_the_lines(ns, kind, over):
+    chain = synth.make_mechanism("h2").nr * (80 + ns)
+    _against_the_oracle(ns, (chain if kind != "analytical" else chain * 11 // 5) + over)
