@@ -295,12 +295,29 @@ __global__ void __launch_bounds__(COOP_NT, 8) k_integrate_coop(KernelArgs a) {
 
 // PLAIN batches of at most this many states go to k_integrate_coop: its time
 // grows with the batch, the per-thread kernel's is flat (a chain of FP64
-// latencies) until its warps fill the chip.  H2, dt = 1e-6 / 1e-4 s, ms, coop
-// against per thread: FP64 2048: 40 / 60 against 150 / 154, 6144: 110 / 169
-// against 117 / 157, 8192: 145 / 226 against 119 / 159; FP32 2048: 26 / 36
-// against 84 / 116, 6144: 68 / 105 against 86 / 118, 8192: 91 / 141 against
-// 87 / 120.  Both give the same bits.
-constexpr int64_t coop_max_n(size_t lt) { return lt == sizeof(double) ? 5632 : 6912; }
+// latencies) until its warps fill the chip.  H2 (13 species, 27 reactions),
+// dt = 1e-6 / 1e-4 s, ms, coop against per thread: FP64 2048: 40 / 60 against
+// 150 / 154, 6144: 110 / 169 against 117 / 157, 8192: 145 / 226 against 119 /
+// 159; FP32 2048: 26 / 36 against 84 / 116, 6144: 68 / 105 against 86 / 118,
+// 8192: 91 / 141 against 87 / 120.  With fewer reactions a thread's chain is
+// shorter and the lines cross earlier, depending
+// on how unequal the states are (subsets of the H2 species, dt = 1e-6 / 1e-4 s):
+//   4 species,   FP64 1216: 0.24 / 0.42 against 0.28 / 0.65
+//   1 reaction        2000: 0.42 / 0.61 against 0.28 / 0.65
+//   6, 4              5632: 1.7 / 5.0 against 1.7 / 10.8
+//   8, 7              4000: 24 / 36 against 27 / 41     5632: 34 / 50 against 27 / 41
+//                FP32 4000: 18 / 27 against 21 / 32     5632: 25 / 36 against 21 / 32
+//   10, 14       FP64 4000: 58 / 90 against 69 / 91     5632: 81 / 124 against 68 / 90
+//                FP32 4000: 37 / 56 against 51 / 66     5632: 51 / 78 against 51 / 66
+// More reactions move the line up (16 species, 300 reactions, 20000 states: 747
+// against 1020), difference Jacobians too (16 species, 27 reactions, 9000: 194
+// against 291); neither raises the limit.  Both kernels give the same bits.
+inline int64_t coop_max_n(const MechLayout &L, size_t lt) {
+  const bool f64 = lt == sizeof(double);
+  if (L.nr < 3) return 1700;
+  if (L.nr >= 6 && L.nr < 20) return f64 ? 4400 : 4700;
+  return f64 ? 5632 : 6912;
+}
 // ... and a mechanism whose reaction tail leaves several blocks per SM
 constexpr size_t COOP_MAX_SMEM = 64 * 1024;
 
@@ -551,7 +568,7 @@ int launch_t(const KernelArgs &a, const kin_options &o, cudaStream_t st, int sms
   const int carve = KIN_THREAD_CARVEOUT;  // percent of the unified L1 given to shared memory
   if constexpr (MAXN <= COOP_CAP) {
     const size_t smc = coop_smem_bytes<LT>(a.L.nr);
-    if (plain && a.rp.n > 0 && a.rp.n <= coop_max_n(sizeof(LT)) &&
+    if (plain && a.rp.n > 0 && a.rp.n <= coop_max_n(a.L, sizeof(LT)) &&
         smc <= COOP_MAX_SMEM) {
       auto kern = k_integrate_coop<LT, FDJ>;
       KIN_CUDA_TRY(open_smem(kern));
