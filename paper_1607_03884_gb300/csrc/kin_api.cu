@@ -969,7 +969,7 @@ static bool chem_on_teams(kin_mech *m, double h, const double *scal, const doubl
   a.hot = m->d_hot;
   a.gslots = INT64_MAX / 8;  // no slots are used
   TeamLaunch g;
-  if (!team_shape(a, a.L.ns, sizeof(float), sms, g)) return false;
+  if (!team_shape(a, a.L.ns, sizeof(float), sms, TEAM_MAX, g)) return false;
   auto kern = k_team_chem<WHAT>;
   rc = KIN_OK;
   if (open_smem(kern) != cudaSuccess) {

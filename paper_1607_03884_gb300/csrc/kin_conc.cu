@@ -157,8 +157,8 @@ struct ConcArgs {
   const double *aw;
 };
 
-template <typename LT>
-__global__ void __launch_bounds__(TEAM_MAX *TEAM_NT, 1) k_integrate_conc(ConcArgs ca) {
+template <typename LT, int TEAMS>
+__global__ void __launch_bounds__(TEAMS *TEAM_NT, 1) k_integrate_conc(ConcArgs ca) {
   using G = Grp<32>;
   extern __shared__ __align__(16) unsigned char team_smem[];
   const KernelArgs &a = ca.a;
@@ -261,8 +261,11 @@ int launch_conc(ConcArgs ca, cudaStream_t st, int sms) {
   KernelArgs &a = ca.a;
   if (!a.gscratch || a.gslots < 1) return KIN_ERR_UNSUPPORTED;
   TeamLaunch g;
-  if (!team_shape(a, ca.N, sizeof(LT), sms, g)) return KIN_ERR_UNSUPPORTED;
-  auto kern = k_integrate_conc<LT>;
+  const int most = team_most(sizeof(LT), false, ca.N, a.rp.n, sms);
+  if (!team_shape(a, ca.N, sizeof(LT), sms, most, g)) return KIN_ERR_UNSUPPORTED;
+  auto kern = k_integrate_conc<LT, TEAM_MAX>;
+  if constexpr (sizeof(LT) == sizeof(float))
+    if (most == TEAM_MANY) kern = k_integrate_conc<LT, TEAM_MANY>;
   KIN_CUDA_TRY(open_smem(kern));
   kern<<<g.grid, g.threads, g.smem, st>>>(ca);
   KIN_CUDA_TRY(cudaGetLastError());

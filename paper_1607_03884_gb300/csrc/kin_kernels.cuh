@@ -419,9 +419,9 @@ __host__ __device__ inline size_t lanes_smem_bytes(const MechLayout &L_, int lan
 }
 
 // WARP layout with 32 lanes: a state per team of three warps (kin_team.cuh),
-// up to four teams per block, one block per SM.
-template <typename LT, bool FDJ>
-__global__ void __launch_bounds__(TEAM_MAX *TEAM_NT, 1) k_integrate_team(KernelArgs a) {
+// up to TEAMS teams per block, one block per SM.
+template <typename LT, bool FDJ, int TEAMS>
+__global__ void __launch_bounds__(TEAMS *TEAM_NT, 1) k_integrate_team(KernelArgs a) {
   using G = Grp<32>;
   extern __shared__ __align__(16) unsigned char team_smem[];
   const MechView m = make_view(a.L, a.tab, a.itab);
@@ -489,13 +489,13 @@ struct TeamLaunch {
 // 24 bytes and 8 per slot and efficiency, beside at most 45 KB of matrices and
 // species vectors.  (Only some 2900 reactions of six slots that change no
 // species at all would not; they are refused.)
-inline bool team_shape(KernelArgs &a, int N, size_t lt, int sms, TeamLaunch &g) {
+inline bool team_shape(KernelArgs &a, int N, size_t lt, int sms, int most, TeamLaunch &g) {
   const size_t budget = BLOCK_SMEM, tb = team_bytes(a.L, N, lt), hot = hot_offsets(a.L).bytes;
   if (!a.hot || tb > budget) return false;
   a.hot_smem = hot + tb <= budget;
   const size_t fixed = a.hot_smem ? hot : 0;
   int64_t teams = (int64_t)((budget - fixed) / tb);
-  teams = teams < TEAM_MAX ? teams : TEAM_MAX;
+  teams = teams < most ? teams : most;
   const int64_t want = (a.rp.n + sms - 1) / sms;  // a small batch spreads over the SMs
   teams = teams < want ? teams : want;
   int64_t grid = (a.rp.n + teams - 1) / teams;
@@ -506,12 +506,24 @@ inline bool team_shape(KernelArgs &a, int N, size_t lt, int sms, TeamLaunch &g) 
   return true;
 }
 
+// most teams per block for n states of N unknowns: the many from two rounds of
+// them on (at 1e-4 s 1500 states of 17 to 24 species were 2 % slower with
+// seven); difference Jacobians, three right-hand sides at a time, keep every
+// warp busy with four (20 species, 10000 states: 283 ms against 288)
+inline int team_most(size_t lt, bool fd, int N, int64_t n, int sms) {
+  return lt == sizeof(float) && !fd && N <= TEAM_MANY_N && n >= 2ll * TEAM_MANY * sms ? TEAM_MANY
+                                                                                    : TEAM_MAX;
+}
+
 template <typename LT, bool FDJ>
 int launch_team(KernelArgs a, cudaStream_t st, int sms) {
   if (!a.gscratch || a.gslots < 1) return KIN_ERR_UNSUPPORTED;
   TeamLaunch g;
-  if (!team_shape(a, a.L.ns, sizeof(LT), sms, g)) return KIN_ERR_UNSUPPORTED;
-  auto kern = k_integrate_team<LT, FDJ>;
+  const int most = team_most(sizeof(LT), FDJ, a.L.ns, a.rp.n, sms);
+  if (!team_shape(a, a.L.ns, sizeof(LT), sms, most, g)) return KIN_ERR_UNSUPPORTED;
+  auto kern = k_integrate_team<LT, FDJ, TEAM_MAX>;
+  if constexpr (sizeof(LT) == sizeof(float) && !FDJ)
+    if (most == TEAM_MANY) kern = k_integrate_team<LT, FDJ, TEAM_MANY>;
   KIN_CUDA_TRY(open_smem(kern));
   kern<<<g.grid, g.threads, g.smem, st>>>(a);
   KIN_CUDA_TRY(cudaGetLastError());

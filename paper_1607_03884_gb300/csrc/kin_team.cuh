@@ -33,7 +33,17 @@
 namespace kin {
 
 constexpr int TEAM_WARPS = 3, TEAM_NT = 32 * TEAM_WARPS;
-constexpr int TEAM_MAX = 4;    // teams per block: 384 threads leave 168 registers each
+// Teams per block.  384 threads leave 168 registers each; 672 leave 80, which
+// FP32 matrices of up to TEAM_MANY_N unknowns live with: their states are small
+// and short of work for three warps, so that four per SM leave the FP64 unit
+// idle once a batch has more.  FP32, dt = 1e-6 s, ms with one warp per state
+// (16 per SM) / four teams / seven: 13 species, 20000 states 296 / 314 / 297,
+// 3000: 51 / 50 / 47; 17 species and 27 reactions, 20000: 315 / 335 / 317, 3000:
+// 54 / 53 / 50, 700: 24 / 15 / 15; 24 species and 100 reactions, 20000: 475 / 388
+// / 381, 3000: 79 / 63 / 61, 700: 36 / 18 / 19; the concentration form of 13
+// species, 10000: 142 / 153 / 143.  Beyond, 40 species: 3000: 130 / 79 / 79; and
+// FP64 matrices lose by the spills (24 species, 20000: 631 / 647, 53: 258 / 275).
+constexpr int TEAM_MAX = 4, TEAM_MANY = 7, TEAM_MANY_N = 24;
 constexpr int TEAM_PANEL = 4;  // columns per factorisation panel
 
 // Rounded products and fused sums, written out where the matrices' bits
@@ -698,7 +708,7 @@ __device__ __forceinline__ void smith_quot(LT a, LT b, LT r, LT den, LT iden, in
 // update the rest, a column per lane.
 template <typename LT, bool PIVOT>
 __device__ __noinline__ int team_lu_cplx(int N, const TeamBuf<LT> &t, int wt) {
-  const int lane = threadIdx.x & 31, ld = t.ld, col = lane + 32 * (wt - 1), bar = t.bar + TEAM_MAX;
+  const int lane = threadIdx.x & 31, ld = t.ld, col = lane + 32 * (wt - 1), bar = t.bar + TEAM_MANY;
   cplx_t<LT> *a = t.E2;
   int src0 = lane, src1 = lane + 32;
   unsigned mode0 = 0, mode1 = 0;
