@@ -23,3 +23,22 @@ def test_moments_of_few_rows(M, d):
     # FP64 sums rounded once to FP32 (2^-24), the deviation's square root too
     np.testing.assert_allclose(mean.cpu().numpy(), x.mean(0), rtol=2e-7)
     np.testing.assert_allclose(std.cpu().numpy(), np.maximum(x.std(0), 1e-12), rtol=4e-7)
+
+
+@pytest.mark.parametrize("n", [99999, 100000, 100001])
+@pytest.mark.parametrize("nz", [1, 27, 28])
+def test_targets_by_rows_and_by_tiles(n, nz):
+    rng = np.random.default_rng(nz)
+    h, z = 10.0 ** rng.uniform(-12, -6, n), rng.standard_normal((nz, n))
+    mu = rng.standard_normal(1 + nz).astype(np.float32)
+    sd = rng.uniform(0.5, 2.0, 1 + nz).astype(np.float32)
+    t = np.concatenate([np.log(h)[:, None], z.T], axis=1)
+    for norm in ((), (_dev(mu), _dev(sd))):
+        tgt = torch.full((n, 1 + nz), np.nan, dtype=torch.float32, device="cuda")
+        kin.targets(nz, _dev(h), _dev(z), tgt, *norm)
+        want = t.astype(np.float32)  # then a difference and a quotient in FP32
+        if norm:
+            want = (want - mu) / sd
+        # log h may round to the neighbouring FP32 value: 2^-23 of |log h| < 28,
+        # over the deviation
+        np.testing.assert_allclose(tgt.cpu().numpy(), want, rtol=1.3e-7, atol=1e-5 if norm else 0)
