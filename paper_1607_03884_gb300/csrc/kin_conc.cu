@@ -373,8 +373,8 @@ extern "C" int kin_conc_create(const kin_mech_desc *desc, kin_conc **out) {
   }
   c->device = dev;
   // one Jacobian slot (with the complex matrix when that is global) per
-  // resident warp: at most 16 whole-warp groups per SM
-  c->gslots = (int64_t)sms * 16;
+  // resident team: one block of them per SM
+  c->gslots = (int64_t)sms * team_slots(N);
   const size_t gbytes =
       (size_t)c->gslots * warp_slot_mats(sizeof(double)) * N * (N + 1) * sizeof(double);
   if (cudaMalloc(&c->d_tab, sizeof(double) * L.nd) != cudaSuccess ||

@@ -515,6 +515,9 @@ inline int team_most(size_t lt, bool fd, int N, int64_t n, int sms) {
                                                                                     : TEAM_MAX;
 }
 
+// workspace slots per SM that teams of N unknowns can use
+inline int team_slots(int N) { return N <= TEAM_MANY_N ? TEAM_MANY : TEAM_MAX; }
+
 template <typename LT, bool FDJ>
 int launch_team(KernelArgs a, cudaStream_t st, int sms) {
   if (!a.gscratch || a.gslots < 1) return KIN_ERR_UNSUPPORTED;
