@@ -22,10 +22,9 @@ namespace {
 // vectors holds phi[var[g]].
 struct ConcStructure {
   int N = 0;
-  int k0 = 0;                 // pivots k0 .. N-1 form a full trailing block
   std::vector<int> var;       // [N] element -> phi index
   std::vector<uint8_t> pat;   // [N*N] filled L + U pattern in element order
-  std::vector<int> lp, li, up, uj, cp, ci;
+  std::vector<int> below, right, above;  // [N] filled entries beside each pivot
   int64_t nnz_J = 0, nnz_LU = 0;
 };
 
@@ -111,26 +110,15 @@ int conc_analyse(const kin_mech_desc *d, ConcStructure &S) {
         if (P[(size_t)k * N + j]) P[(size_t)i * N + j] = 1;
     }
   for (uint8_t x : P) S.nnz_LU += x;
-  S.lp.assign(1, 0);
-  S.up.assign(1, 0);
-  S.cp.assign(1, 0);
-  for (int k = 0; k < N; ++k) {
-    for (int i = k + 1; i < N; ++i)
-      if (P[(size_t)i * N + k]) S.li.push_back(i);
-    for (int j = k + 1; j < N; ++j)
-      if (P[(size_t)k * N + j]) S.uj.push_back(j);
-    for (int i = 0; i < k; ++i)
-      if (P[(size_t)i * N + k]) S.ci.push_back(i);
-    S.lp.push_back((int)S.li.size());
-    S.up.push_back((int)S.uj.size());
-    S.cp.push_back((int)S.ci.size());
-  }
-  S.k0 = N;
-  for (int k = N - 1; k >= 0; --k) {
-    const int l = S.lp[k + 1] - S.lp[k], u = S.up[k + 1] - S.up[k];
-    if (l != N - 1 - k || u != N - 1 - k) break;
-    S.k0 = k;
-  }
+  S.below.assign(N, 0);
+  S.right.assign(N, 0);
+  S.above.assign(N, 0);
+  for (int k = 0; k < N; ++k)
+    for (int i = 0; i < N; ++i) {
+      if (i > k) S.below[k] += P[(size_t)i * N + k];
+      if (i > k) S.right[k] += P[(size_t)k * N + i];
+      if (i < k) S.above[k] += P[(size_t)i * N + k];
+    }
   return KIN_OK;
 }
 
@@ -140,9 +128,9 @@ int conc_analyse(const kin_mech_desc *d, ConcStructure &S) {
 void conc_counts(const ConcStructure &S, int64_t *out) {
   int64_t lu = 0, sol = S.N;
   for (int k = 0; k < S.N; ++k) {
-    const int64_t l = S.lp[k + 1] - S.lp[k], u = S.up[k + 1] - S.up[k];
+    const int64_t l = S.below[k], u = S.right[k];
     lu += 1 + l + 2 * l * u;
-    sol += 2 * l + 2 * (S.cp[k + 1] - S.cp[k]);
+    sol += 2 * l + 2 * S.above[k];
   }
   out[0] = S.nnz_J;
   out[1] = S.nnz_LU;
