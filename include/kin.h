@@ -93,19 +93,23 @@ typedef struct kin_mech kin_mech;
 /* Kernel layouts. */
 enum {
   KIN_LAYOUT_PLAIN = 0, /* one state per thread, nested step/Newton loops: the
-                           paper's GPU organisation (Sec. 1, Sec. 3.3) */
+                           paper's GPU organisation (Sec. 1, Sec. 3.3).  Small
+                           batches of up to 16 species (a few thousand
+                           states, fewer for few reactions) run one state
+                           per block of 96 threads, with the same bits */
   KIN_LAYOUT_QUEUE = 1  /* one state per thread in a persistent launch: every
                            loop trip is one step attempt per lane, and a lane
                            whose state is done takes the next one from an
                            atomic work queue (answers the warp divergence of
                            Sec. 3.3: no lane waits for the slowest state) */,
-  KIN_LAYOUT_WARP = 2,  /* one state per group of kin_options.lanes lanes
-                           (a whole warp: ns <= 63; 4, 8 or 16 lanes:
-                           ns <= 15): vectors over the group's lanes, Newton
-                           matrices in shared memory, group-cooperative LU
-                           and solves, rates in parallel over reactions;
-                           groups pop states from the atomic queue (the
-                           per-block strategy of Sec. 3.3) */
+  KIN_LAYOUT_WARP = 2,  /* one state per group of kin_options.lanes lanes (32:
+                           ns <= 63; 4, 8 or 16: ns <= 15): vectors over the
+                           lanes of a warp, Newton matrices in shared memory,
+                           group-cooperative LU and solves, rates in parallel
+                           over reactions; with 32 lanes two more warps share
+                           the state's work (a team of 96 threads).  Groups
+                           pop states from the atomic queue (the per-block
+                           strategy of Sec. 3.3) */
   KIN_LAYOUT_AUTO = 3   /* the library chooses at each call: the launch
                            configuration kin_autotune last found for this
                            mechanism with the same matrix precision, Jacobian
@@ -126,7 +130,9 @@ typedef struct {
   int32_t jac_fd;        /* 1: CVODE-style one-sided difference Jacobian   (0) */
   int32_t max_steps;     /* internal step limit per state             (100000) */
   int32_t nit;           /* Newton iterations per step                     (7) */
-  int32_t block;         /* threads per block; 0 = library choice          (0) */
+  int32_t block;         /* PLAIN, QUEUE: threads per block, 32 or 64; 0 =
+                            library choice.  Without effect where PLAIN runs
+                            one state per block                           (0) */
   int32_t grid_per_sm;   /* QUEUE: resident blocks per SM; 0 = occupancy   (0) */
   int32_t transform_tol; /* 1: rtol' = 0.1 rtol^(2/3), atol' = rtol' atol/rtol (1) */
   int32_t queue_refill;  /* QUEUE: a warp refills once at least this many of its
@@ -150,7 +156,8 @@ typedef struct {
                             n <= 2^31 - 1 with an order.              (NULL) */
   int32_t lanes;         /* KIN_LAYOUT_WARP: lanes per state, 4, 8, 16 or 32
                             (0 = 32).  4, 8 and 16 hold at most 15 species
-                            and place 32/lanes states in each warp      (0) */
+                            and place 32/lanes states in each warp; 32 is a
+                            team of three warps per state                (0) */
   double h_fixed;        /* > 0: constant internal step h_fixed (the last step
                             clipped onto dt; x + 1.0001 h >= dt ends it),
                             every step accepted, a fresh Jacobian every step,
@@ -281,7 +288,9 @@ int kin_order_states(kin_mech *m, const double *Y, const double *T, const double
 
 /* Source terms f(y) for n states (y = [T, Y_0..Y_{ns-2}], N = ns):
  * y dev [N][n], P dev [n], f dev [N][n] out.  Unit-level entry of the
- * right-hand side every Radau stage evaluates (Sec. 2.1). */
+ * right-hand side every Radau stage evaluates (Sec. 2.1).  Beyond 16 species
+ * the kernel follows the batch size (a state per warp, or per thread for some
+ * thousand states and more), and with it the last bits; kin_jacobian's too. */
 int kin_rhs(kin_mech *m, const double *y, const double *P, int64_t n, double *f, void *stream);
 
 /* Jacobian df/dy for n states: J dev [N*N][n] out, entry (r, c) at
@@ -305,17 +314,18 @@ int kin_jacobian(kin_mech *m, const double *y, const double *P, int64_t n, int32
  * the process exits) instead of a kin_mech's workspace.  The paper has no
  * counterpart.  Y, T, P and status are as for kin_integrate_ex (dev
  * pointers).
- *   - Kernel: one state per thread (PLAIN), FP64 Newton matrices, whatever
- *     the mechanism size: the state-per-warp layout needs a per-mechanism
- *     workspace.  It serves mechanisms of up to 16 species at the thread
- *     layouts' speed; larger ones are integrated correctly but far more
- *     slowly than kin_integrate_ex would (its 64-species per-thread kernel).
+ *   - Kernel: PLAIN, FP64 Newton matrices, whatever the mechanism size: the
+ *     WARP layout needs a per-mechanism workspace.  It serves mechanisms of
+ *     up to 16 species at that layout's speed; larger ones are integrated
+ *     correctly but far more slowly than kin_integrate_ex would (its
+ *     64-species per-thread kernel).
  *   - Set-up: the first call on a device looks up the array's device
- *     address.  The first launch of an integration kernel on a device can
- *     also make the CUDA driver reserve local memory for the kernel's
- *     per-thread frame times the device's resident threads (gigabytes for
- *     these kernels); a host whose allocator reserves all device memory
- *     should make one call, on any small batch, before it does.
+ *     address.  It also makes the CUDA driver reserve local memory for the
+ *     per-thread kernels' frames times the device's resident threads
+ *     (gigabytes), whatever its own batch, for mechanisms of up to 16 species
+ *     and, at the first call with a larger one, for those; a host whose
+ *     allocator reserves all device memory should make one call, on any small
+ *     batch, before it does.
  *   - Not capturable: the tables are uploaded from host memory the call
  *     frees, so a call on a stream that is being captured into a CUDA graph
  *     returns KIN_ERR_UNSUPPORTED and issues nothing.
@@ -424,15 +434,15 @@ int kin_conc_get_stats(kin_conc *c, int64_t *out);
  * (Arnoldi), grown until Saad's leading error term of every product taken
  * from it is at most kappa in the step's error weights (kappa = 0: the
  * whole space), and phi_k of the small Hessenberg matrix from the
- * exponential of an augmented matrix (scaling and squaring, Pade (6,6)).
- * One state per warp; ns <= 57.
+ * scaled matrix by doublings of exp - I and the phi blocks together.
+ * One state per warp; ns <= 58.
  * ------------------------------------------------------------------------- */
 typedef struct kin_exprb kin_exprb;
 
 /* Build the tables and the per-warp workspace (basis, Hessenberg and
- * matrix-function work, about 8 (ns+7)^2 doubles per resident warp) on the
+ * matrix-function work, about 9 ns (ns+2) doubles per resident warp) on the
  * current device.  Errors: those of kin_mech_create; KIN_ERR_UNSUPPORTED
- * for ns > 57. */
+ * for ns > 58. */
 int kin_exprb_create(const kin_mech_desc *desc, kin_exprb **out);
 
 /* Free (NULL is ignored; no work may be in flight). */
@@ -460,8 +470,7 @@ int kin_exprb_get_stats(kin_exprb *x, int64_t *out);
  * testing: out[i*p + k-1] = (phi_k(tau H) e1)_i for k = 1..p, i < m, H dev
  * [m*m] row-major, out dev [m*p]; 1 <= m <= ns, 1 <= p <= 5.  Runs on one
  * warp in the first workspace slot (no integration may be in flight).
- * KIN_ERR_INVALID_ARG outside those ranges; NaN when the Pade denominator is
- * singular or tau H is not finite. */
+ * KIN_ERR_INVALID_ARG outside those ranges; NaN when tau H is not finite. */
 int kin_exprb_phi(kin_exprb *x, const double *H, int32_t m, int32_t p, double tau, double *out,
                   void *stream);
 
