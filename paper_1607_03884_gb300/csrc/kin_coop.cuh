@@ -15,9 +15,9 @@
 // the complex linear algebra on different warps, the complex substitution's
 // real and imaginary parts on different lanes; everything lives in shared
 // memory.  Measured (FP64, dt = 1e-6 s): 33 states 123 -> 9.3 ms, 1024 states
-// 153 -> 20.7 ms.  What is left on one state: 35 % chemistry (the Troe branch
-// and the logarithms), 25 % substitutions (78 dependent terms), 15 %
-// factorisations, the rest scalar control and norms.
+// 153 -> 20.7 ms.  What is left on one state is its dependent chain: the Troe
+// branch and the logarithms, 78 terms per back substitution, the pivots, scalar
+// control and norms.
 //
 // Every element is computed by the expressions of kin_device.cuh and
 // kin_radau.cuh and every sum runs over its terms in the same order, so the

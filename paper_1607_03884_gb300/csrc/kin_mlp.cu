@@ -44,7 +44,10 @@ __device__ __forceinline__ float silu_grad(float a) {
 
 // ---------------------------------------------------------------------------
 // GEMM, generic strides: C[m][n] (+)= sum_k A(m,k) B(k,n) with
-// A(m,k) = A[m*sam + k*sak], B(k,n) = B[k*sbk + n*sbn]; out of range = 0.
+// A(m,k) = A[m*sam + k*sak], B(k,n) = B[k*sbk + n*sbn]; out of range = 0.  It
+// serves the weight gradients, and every product of widths that are not
+// multiples of 8 (the others' forward and input-gradient products are
+// k_gemm_kk's below).
 //
 // BF16 version on the 5th-generation tensor cores (tcgen05): a CTA of four
 // warps owns a 128 x 128 tile of C.  Per 64-wide slice of K, the warps copy
@@ -58,8 +61,8 @@ __device__ __forceinline__ float silu_grad(float a) {
 // lanes 32w..32w+31, the tile's rows) and writes or adds C.  Every wait is
 // bounded: on expiry the kernel sets *err, waits (bounded) for its MMAs and
 // loads, frees its TMEM and returns.
-// A K-contiguous operand with 16-byte rows (the forward pass and the input
-// gradients) is loaded by the tensor memory accelerator instead: one thread
+// A K-contiguous operand with 16-byte rows (the input layer and the output
+// layer's input gradient) is loaded by the tensor memory accelerator: one thread
 // issues eight cp.async.bulk.tensor boxes of 8 K x 128 rows per slice, each
 // landing as 16 core matrices in a row (core (g, c) at c * 2048 + g * 128
 // bytes), completion counted in bytes on a second mbarrier; the TMA fills
