@@ -300,8 +300,8 @@ __global__ void __launch_bounds__(COOP_NT, 8) k_integrate_coop(KernelArgs a) {
 // 150 / 154, 6144: 110 / 169 against 117 / 157, 8192: 145 / 226 against 119 /
 // 159; FP32 2048: 26 / 36 against 84 / 116, 6144: 68 / 105 against 86 / 118,
 // 8192: 91 / 141 against 87 / 120.  With fewer reactions a thread's chain is
-// shorter and the lines cross earlier, depending
-// on how unequal the states are (subsets of the H2 species, dt = 1e-6 / 1e-4 s):
+// shorter and the lines cross earlier, depending on how unequal the states are
+// (subsets of the H2 species, dt = 1e-6 / 1e-4 s):
 //   4 species,   FP64 1216: 0.24 / 0.42 against 0.28 / 0.65
 //   1 reaction        2000: 0.42 / 0.61 against 0.28 / 0.65
 //   6, 4              5632: 1.7 / 5.0 against 1.7 / 10.8
